@@ -36,23 +36,9 @@
 
 #include "glz_common.h"
 #include "glz_device.cuh"
+#include "mask_parse.cuh"
 
 namespace glz {
-
-template <int S>
-struct SymType;
-template <>
-struct SymType<1> {
-  using T = uint8_t;
-};
-template <>
-struct SymType<2> {
-  using T = uint16_t;
-};
-template <>
-struct SymType<4> {
-  using T = uint32_t;
-};
 
 constexpr uint16_t kNoPos = 0xFFFF;  // chunk positions are < 32768
 
@@ -1004,7 +990,8 @@ __device__ __forceinline__ void write_header(const BufDesc &B, uint32_t lane) {
 // Steps 1-6 for chunk c of buffer B (item `item` of a batch).  Returns false
 // when the TMA copy never landed (the warp must stop: its barrier phase is
 // unknown; the chunk was still published so no other warp waits on it).
-template <int S, int NJ, bool WIDE>
+// MASK: the parse by equality masks (NJ words per mask), else hash chains.
+template <int S, int NJ, bool WIDE, bool MASK>
 __device__ __forceinline__ bool compress_chunk(const CompressArgs &A, const BufDesc &B,
                                                uint32_t item, uint32_t c, WarpState &W,
                                                uint32_t lane) {
@@ -1053,42 +1040,49 @@ __device__ __forceinline__ bool compress_chunk(const CompressArgs &A, const BufD
   if (S >= 2 && W.try_literal && bm_words >= 16 && 4 * bm_words >= k)
     literal = literal_chunk<S>(sym, k, B, reinterpret_cast<uint32_t *>(W.links_base), bm_words,
                                W.maybe, lane);
-  uint32_t marked = 0;
-  if (!literal) {
-    build_chains<S, WIDE>(sym, k, B, A.sm, reinterpret_cast<uint16_t *>(W.pay), W.maybe,
-                          links, lane);
-    for (uint32_t i = lane; i < (k + 31) / 32; i += 32) marked |= W.maybe[i];
-  }
-  __syncwarp();
-
-  // 3. greedy parse: the walk records the pointers (a bitmap in the flags
-  // area, their payload bytes listed in the payload area).  With no marked
-  // position, or no pointer, the record is k literals: zero flags, then the
-  // staged chunk itself.
+  // 3. greedy parse.  By masks: the record itself, in shared memory.  By
+  // chains: the walk records the pointers (a bitmap in the flags area, their
+  // payload bytes listed in the payload area).  With no marked position, or
+  // no pointer, the record is k literals: zero flags, then the staged chunk
+  // itself.
+  const uint32_t tail = bytes - k * S;
   uint32_t ntok = k, pb = k * S, np = 0;
   bool sane = true;
   const uint8_t *payload = W.inb;
   uint32_t *pbits = reinterpret_cast<uint32_t *>(W.flags);
-  if (__any_sync(kFull, marked != 0)) {
-    greedy_walk<S, NJ, WIDE>(sym, k, B, A.sm, W.maybe, links, pbits, W.pay, lane, ntok, pb,
-                             np, sane);
-    if (!sane) {
-      if (lane == 0) atomicOr(A.err, kErrInternal);
-      ntok = k;
-      pb = k * S;
-      np = 0;
+  if constexpr (MASK) {
+    if (!literal)
+      mask_parse<S, NJ>(W.inb, k, tail, B, reinterpret_cast<uint32_t *>(W.links_base),
+                        reinterpret_cast<uint32_t *>(W.pay), pbits,
+                        A.sm.pay_off - A.sm.flags_off, lane, ntok, pb, np);
+  } else {
+    uint32_t marked = 0;
+    if (!literal) {
+      build_chains<S, WIDE>(sym, k, B, A.sm, reinterpret_cast<uint16_t *>(W.pay), W.maybe,
+                            links, lane);
+      for (uint32_t i = lane; i < (k + 31) / 32; i += 32) marked |= W.maybe[i];
+    }
+    __syncwarp();
+    if (__any_sync(kFull, marked != 0)) {
+      greedy_walk<S, NJ, WIDE>(sym, k, B, A.sm, W.maybe, links, pbits, W.pay, lane, ntok, pb,
+                               np, sane);
+      if (!sane) {
+        if (lane == 0) atomicOr(A.err, kErrInternal);
+        ntok = k;
+        pb = k * S;
+        np = 0;
+      }
     }
   }
   // the record: 0 = zero flags + the staged chunk (all literals) or the
   // chunk alone (stored); 1 = pointers, emitted at the record's place;
   // 2 = pointers, emitted into shared memory (flags over the bitmap,
   // payload over the staged chunk)
-  uint32_t kind = np != 0 ? 1u : 0u;
+  uint32_t kind = np != 0 ? (MASK ? 2u : 1u) : 0u;
   W.try_literal = kind == 0;
   // 4. stream version 2, last chunk: the 1..S-1 bytes after the last whole
   // symbol follow the tokens as they are (in the staged chunk they already
   // follow the k symbols)
-  const uint32_t tail = bytes - k * S;
   pb += tail;
   uint32_t fb = (ntok + 7) / 8;
   if (B.version == 2 && fb + pb >= bytes) {
@@ -1098,6 +1092,12 @@ __device__ __forceinline__ bool compress_chunk(const CompressArgs &A, const BufD
     fb = 0;
     pb = bytes;
     payload = W.inb;
+    if (kind == 2) {  // the mask parse wrote over the chunk: read it again
+      if (B.in_aligned) warp_copy(W.inb, src, bytes, lane);
+      else
+        for (uint32_t i = lane; i < bytes; i += 32) W.inb[i] = src[i];
+      __syncwarp();
+    }
     kind = 0;
   }
   if (kind == 1 && S * B.m >= 1 + B.offB) {
@@ -1169,9 +1169,17 @@ __device__ __forceinline__ uint32_t take_ticket(const CompressArgs &A, uint32_t 
   return __shfl_sync(kFull, t, 0);
 }
 
+// Register limit of a kernel, as resident blocks of 256 threads: the mask
+// parse left alone takes 140 registers, far past what the shared memory
+// would keep resident (28 warps per SM at C = 4096, S = 2; 23 at C = 4096,
+// S = 4, W = 256; 15 at C = 8192, W = 512).
+constexpr int min_blocks(int nj, bool mask) {
+  return mask ? (nj <= 4 ? 4 : nj <= 8 ? 3 : 2) : (nj < 32 ? 4 : 3);
+}
+
 // Single buffer: the symbol size is a template parameter.
-template <int S, int NJ>
-__global__ void __launch_bounds__(256) compress_kernel(const CompressArgs A) {
+template <int S, int NJ, bool MASK>
+__global__ void __launch_bounds__(256, min_blocks(NJ, MASK)) compress_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31;
   WarpState W;
@@ -1180,7 +1188,7 @@ __global__ void __launch_bounds__(256) compress_kernel(const CompressArgs A) {
     const uint32_t c = take_ticket(A, lane);
     if (c >= A.end_chunk) break;
     // one-byte links exactly when W <= 256, which is when NJ <= 8
-    if (!compress_chunk<S, NJ, (NJ > 8)>(A, A.buf, 0, c, W, lane)) break;
+    if (!compress_chunk<S, NJ, (NJ > 8), MASK>(A, A.buf, 0, c, W, lane)) break;
   }
   drain_parked(A, W, true, lane);
   if (lane == 0) checked_fold(A.err);
@@ -1203,10 +1211,31 @@ __device__ __forceinline__ uint32_t find_item(const CompressArgs &A, uint64_t g,
   return lo;
 }
 
+// A chunk of a batch, by its buffer's symbol size.  (Out of line: one copy
+// of each variant, whatever the number of kernels.)
+template <int S, int NJ, bool WIDE, bool MASK>
+__device__ __noinline__ bool batch_chunk(const CompressArgs &A, const BufDesc &item_desc,
+                                         uint32_t item, uint32_t c, WarpState &W, uint32_t lane) {
+  const BufDesc B = item_desc;
+  return compress_chunk<S, NJ, WIDE, MASK>(A, B, item, c, W, lane);
+}
+
+template <int NJ, bool WIDE, bool MASK>
+__device__ __forceinline__ bool compress_item(const CompressArgs &A, const BufDesc &B,
+                                              uint32_t item, uint32_t c, WarpState &W,
+                                              uint32_t lane) {
+  switch (B.S) {
+    case 1: return batch_chunk<1, NJ, WIDE, MASK>(A, B, item, c, W, lane);
+    case 2: return batch_chunk<2, NJ, WIDE, MASK>(A, B, item, c, W, lane);
+    default: return batch_chunk<4, NJ, WIDE, MASK>(A, B, item, c, W, lane);
+  }
+}
+
 // Batch: work items are the chunks of all buffers in order; each buffer
 // carries its own parameters, so the symbol size is dispatched per chunk.
 template <int NJ>
-__global__ void __launch_bounds__(256) compress_batch_kernel(const CompressArgs A) {
+__global__ void __launch_bounds__(256, min_blocks(NJ, true))
+    compress_batch_kernel(const __grid_constant__ CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31;
   WarpState W;
@@ -1218,26 +1247,15 @@ __global__ void __launch_bounds__(256) compress_batch_kernel(const CompressArgs 
     const BufDesc B = A.items[item];
     const uint32_t c = static_cast<uint32_t>(g - B.gbase);
     bool ok;
-    if constexpr (NJ > 8) {
-      if (B.W > 256) {
-        switch (B.S) {
-          case 1: ok = compress_chunk<1, NJ, true>(A, B, item, c, W, lane); break;
-          case 2: ok = compress_chunk<2, NJ, true>(A, B, item, c, W, lane); break;
-          default: ok = compress_chunk<4, NJ, true>(A, B, item, c, W, lane); break;
-        }
-      } else {
-        switch (B.S) {
-          case 1: ok = compress_chunk<1, NJ, false>(A, B, item, c, W, lane); break;
-          case 2: ok = compress_chunk<2, NJ, false>(A, B, item, c, W, lane); break;
-          default: ok = compress_chunk<4, NJ, false>(A, B, item, c, W, lane); break;
-        }
-      }
+    if (mask_parse_takes(B.S, B.W, B.m, B.match)) {
+      // (an instance for each class of windows: a mask word costs every position)
+      if (NJ <= 4 || B.W <= 128) ok = compress_item<4, false, true>(A, B, item, c, W, lane);
+      else if (NJ <= 8 || B.W <= 256) ok = compress_item<8, false, true>(A, B, item, c, W, lane);
+      else ok = compress_item<16, false, true>(A, B, item, c, W, lane);
+    } else if (NJ <= 8 || B.W <= 256) {
+      ok = compress_item<(NJ < 8 ? NJ : 8), false, false>(A, B, item, c, W, lane);
     } else {
-      switch (B.S) {
-        case 1: ok = compress_chunk<1, NJ, false>(A, B, item, c, W, lane); break;
-        case 2: ok = compress_chunk<2, NJ, false>(A, B, item, c, W, lane); break;
-        default: ok = compress_chunk<4, NJ, false>(A, B, item, c, W, lane); break;
-      }
+      ok = compress_item<NJ, true, false>(A, B, item, c, W, lane);
     }
     if (!ok) break;
   }

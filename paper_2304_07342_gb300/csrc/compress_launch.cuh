@@ -1,4 +1,4 @@
-// compress_launch.cuh -- host-side launch of compress_kernel<S, NJ>:
+// compress_launch.cuh -- host-side launch of compress_kernel<S, NJ, MASK>:
 // dynamic shared-memory opt-in, occupancy-sized persistent grid.
 #pragma once
 
@@ -9,10 +9,10 @@
 
 namespace glz {
 
-template <int S, int NJ>
+template <int S, int NJ, bool MASK>
 static cudaError_t launch_compress_nj(const CompressArgs &A, int block, unsigned grid_req,
                                       cudaStream_t stream) {
-  auto kern = compress_kernel<S, NJ>;
+  auto kern = compress_kernel<S, NJ, MASK>;
   const size_t smem = static_cast<size_t>(A.sm.per_warp) * (block / 32);
   static LaunchCache lc;
   int per_sm = 0, sms = 0;
@@ -27,16 +27,25 @@ static cudaError_t launch_compress_nj(const CompressArgs &A, int block, unsigned
   return cudaGetLastError();
 }
 
+template <int S, int NJ>
+static cudaError_t launch_compress_mode(const CompressArgs &A, int block, unsigned grid,
+                                        cudaStream_t stream) {
+  if constexpr (32 * NJ <= kMaskMaxWindow)
+    if (mask_parse_takes(S, A.buf.W, A.buf.m, A.buf.match))
+      return launch_compress_nj<S, NJ, true>(A, block, grid, stream);
+  return launch_compress_nj<S, NJ, false>(A, block, grid, stream);
+}
+
 template <int S>
 static cudaError_t launch_compress_t(const CompressArgs &A, uint32_t nj,
                                      int block, unsigned grid, cudaStream_t stream) {
   switch (nj) {
-    case 1: return launch_compress_nj<S, 1>(A, block, grid, stream);
-    case 2: return launch_compress_nj<S, 2>(A, block, grid, stream);
-    case 4: return launch_compress_nj<S, 4>(A, block, grid, stream);
-    case 8: return launch_compress_nj<S, 8>(A, block, grid, stream);
-    case 16: return launch_compress_nj<S, 16>(A, block, grid, stream);
-    case 32: return launch_compress_nj<S, 32>(A, block, grid, stream);
+    case 1: return launch_compress_mode<S, 1>(A, block, grid, stream);
+    case 2: return launch_compress_mode<S, 2>(A, block, grid, stream);
+    case 4: return launch_compress_mode<S, 4>(A, block, grid, stream);
+    case 8: return launch_compress_mode<S, 8>(A, block, grid, stream);
+    case 16: return launch_compress_mode<S, 16>(A, block, grid, stream);
+    case 32: return launch_compress_mode<S, 32>(A, block, grid, stream);
     default: return cudaErrorInvalidValue;
   }
 }

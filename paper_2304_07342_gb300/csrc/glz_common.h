@@ -27,13 +27,36 @@ constexpr uint32_t kErrInternal = 1u << 3;  // a device consistency check failed
 // raises kErrTimeout instead of hanging the GPU.
 constexpr uint32_t kSpinLimit = 1u << 22;
 
+// The parse by equality masks (mask_parse.cuh) takes the exact matchers when
+// records can be written over the staged chunk (S * m >= 1 + offB), the first
+// m rows of any position lie in the two slabs kept (m <= 32) and the window
+// fits the widest instance (512 symbols: 16 mask words per lane; 32 would not
+// leave registers for more than a few warps).  Everything else (the paper's
+// matcher, other sizes) takes the hash chains.
+constexpr uint32_t kMaskMaxWindow = 512;
+__host__ __device__ inline bool mask_parse_takes(uint32_t S, uint32_t W, uint32_t m,
+                                                 uint32_t match) {
+  return match != kMatchPaper && W <= kMaskMaxWindow && m <= 32 &&
+         S * m >= 1u + (W <= 256 ? 1u : 2u);
+}
+// Plane words of one slab of 32 symbols (one per symbol bit) and, for windows
+// of 32 * nw symbols, the planes kept and the rows of two slabs and a spare
+// one (bytes).
+__host__ __device__ constexpr uint32_t mask_plane_words(uint32_t S) { return 8 * S; }
+__host__ __device__ constexpr uint32_t mask_planes_bytes(uint32_t S, uint32_t nw) {
+  return 2 * nw * mask_plane_words(S) * 4;
+}
+__host__ __device__ constexpr uint32_t mask_rows_bytes(uint32_t nw) {
+  return (65 * nw * 4 + 15) & ~15u;
+}
+
 // Per-warp shared-memory layout of the compressor (byte offsets from the
 // warp's slice; every region 16-byte aligned).
 struct CompressSmem {
   uint32_t in_off;     // staged chunk, C bytes
-  uint32_t prev_off;   // u16 per position: previous position, same key hash
+  uint32_t prev_off;   // chain links; or the bit planes of the mask parse
   uint32_t flags_off;  // flag bits of up to k tokens
-  uint32_t pay_off;    // payload staging (worst case); also the hash table
+  uint32_t pay_off;    // hash table, then the pointer list; or the mask parse's rows
   uint32_t pay_bytes;  // size of the payload staging region
   uint32_t maybe_off;  // one bit per position: a match of >= m may exist
   uint32_t mbar_off;   // mbarrier for the TMA bulk copy

@@ -129,8 +129,15 @@ bool params_ok(const lz_params *p) {
   return true;
 }
 
-// Shared-memory slice of one compressing warp.
-glz::CompressSmem compress_layout(const lz_params *p) {
+// The kernels' matcher of an lz_match.
+uint32_t kernel_match(uint32_t match) {
+  return match == LZ_MATCH_PAPER     ? glz::kMatchPaper
+         : match == LZ_MATCH_OVERLAP ? glz::kMatchOverlap
+                                     : glz::kMatchExact;
+}
+
+// Shared-memory slice of one compressing warp (`match`: the kernels').
+glz::CompressSmem compress_layout(const lz_params *p, uint32_t match) {
   const uint32_t S = p->symbol_bytes, C = p->chunk_bytes;
   const uint32_t k = C / S;
   const uint32_t offB = off_bytes(p->window);
@@ -140,20 +147,16 @@ glz::CompressSmem compress_layout(const lz_params *p) {
   uint32_t at = 0;
   sm.in_off = at;
   at += round16(C);
-  sm.prev_off = at;
-  at += round16((p->window > 256 ? 2ull : 1ull) * k);
-  sm.flags_off = at;
-  at += round16(div_up(k, 32) * 4);
-  sm.pay_off = at;
-  // The payload area holds the hash table while the chains are built, then
-  // the pointer list of the walk (1 + offB bytes per pointer, at most k / m
-  // of them); records are emitted in place or at their destination.  For 1-
-  // and 2-byte symbols it takes a table of a quarter as many buckets as the
-  // chunk has positions (or the list, if larger): less shared memory per
-  // warp, more warps resident.
+  // Links of the hash chains, the flags, and the payload area: the hash
+  // table while the chains are built, then the pointer list of the walk
+  // (1 + offB bytes per pointer, at most k / m of them); records are emitted
+  // in place or at their destination.  For 1- and 2-byte symbols it takes a
+  // table of a quarter as many buckets as the chunk has positions (or the
+  // list, if larger): less shared memory per warp, more warps resident.
   // For 4-byte symbols it keeps the size of a worst-case payload, which the
   // literal pre-check's Bloom filter uses (with links and flags) to hold
-  // about 10 bits per position.
+  // about 40 bits per position.
+  uint32_t links = round16((p->window > 256 ? 2ull : 1ull) * k);
   uint32_t pay_region = round16(pay_bytes + 16);
   if (S <= 2) {
     uint32_t lgk = 1;
@@ -163,6 +166,23 @@ glz::CompressSmem compress_layout(const lz_params *p) {
     const uint64_t table = 2ull << lgt;
     pay_region = round16((list > table ? list : table) + 16);
   }
+  if (glz::mask_parse_takes(S, p->window, p->min_match, match)) {
+    // Bit planes in place of the links and rows in place of the payload area.
+    // 1-byte symbols have no literal pre-check and take no more than these:
+    // 14 KiB instead of 34 per warp at C = 8192, W = 512, 15 warps resident
+    // per SM instead of 6.  Others keep the chains' space (with one-byte
+    // links) for the pre-check's bitmap.
+    uint32_t nw = 4;  // (a batch runs small windows with 4 words)
+    while (32 * nw < p->window) nw *= 2;
+    const uint32_t planes = glz::mask_planes_bytes(S, nw), rows = glz::mask_rows_bytes(nw);
+    links = S == 1 ? planes : std::max(planes, round16(k));
+    pay_region = S == 1 ? rows : std::max(rows, pay_region);
+  }
+  sm.prev_off = at;
+  at += links;
+  sm.flags_off = at;
+  at += round16(div_up(k, 32) * 4);
+  sm.pay_off = at;
   sm.pay_bytes = pay_region;
   at += pay_region;
   sm.maybe_off = at;
@@ -396,7 +416,7 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
                                           p->min_match, p->max_match, C,
                                           p->window, out_bytes, st));
 
-  glz::CompressSmem sm = compress_layout(p);
+  glz::CompressSmem sm = compress_layout(p, kernel_match(match));
   if (static_cast<int64_t>(sm.per_warp) > ctx->smem_optin) return LZ_ERR_INVALID_ARG;
   int block = 32;
   int64_t best_blocks = 1;
@@ -437,9 +457,7 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
   A.buf.nc = static_cast<uint32_t>(nc);
   A.buf.records_at = records_at;
   A.buf.in_aligned = (reinterpret_cast<uintptr_t>(d_in) % 16) == 0;
-  A.buf.match = match == LZ_MATCH_PAPER     ? glz::kMatchPaper
-                : match == LZ_MATCH_OVERLAP ? glz::kMatchOverlap
-                                            : glz::kMatchExact;
+  A.buf.match = kernel_match(match);
   A.buf.version = version;
   A.buf.gbase = 0;
   A.total_chunks = nc;
@@ -874,7 +892,7 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
     return cuda_status(glz::launch_header(static_cast<uint8_t *>(d_out), 1u, S, offB,
                                           p->min_match, p->max_match, C, p->window,
                                           out_bytes, st));
-  const glz::CompressSmem sm = compress_layout(p);
+  const glz::CompressSmem sm = compress_layout(p, glz::kMatchExact);
   if (static_cast<int64_t>(sm.per_warp) > nd->smem_optin) return LZ_ERR_INVALID_ARG;
   int block = 32;
   int64_t best_blocks = 1;
@@ -1003,10 +1021,10 @@ lz_status batch_upload(lz_batch *b, int slot, const std::vector<T> &v, const T *
 
 // Per-warp slice covering every parameter set of a batch: each region at its
 // largest size.
-glz::CompressSmem compress_layout_max(const std::vector<lz_params> &ps) {
+glz::CompressSmem compress_layout_max(const std::vector<lz_params> &ps, uint32_t match) {
   uint64_t in = 16, links = 16, flags = 16, pay = 16, maybe = 16;
   for (const lz_params &p : ps) {
-    const glz::CompressSmem one = compress_layout(&p);
+    const glz::CompressSmem one = compress_layout(&p, match);
     in = std::max<uint64_t>(in, one.prev_off - one.in_off);
     links = std::max<uint64_t>(links, one.flags_off - one.prev_off);
     flags = std::max<uint64_t>(flags, one.pay_off - one.flags_off);
@@ -1087,7 +1105,7 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
     while (32 * j < p->window) j *= 2;
     nj = std::max(nj, j);
   }
-  glz::CompressSmem sm = ps.empty() ? glz::CompressSmem{} : compress_layout_max(ps);
+  glz::CompressSmem sm = ps.empty() ? glz::CompressSmem{} : compress_layout_max(ps, match);
   if (!ps.empty() && static_cast<int64_t>(sm.per_warp) > ctx->smem_optin)
     return LZ_ERR_INVALID_ARG;
   int block = 32;
@@ -1428,7 +1446,7 @@ lz_status lz_autotune_ex(lz_ctx *ctx, const void *d_sample, uint64_t sample_byte
     for (lz_tune_trial &t : shape) {
       if (s != LZ_OK) break;
       if (t.warps_per_block &&
-          static_cast<int64_t>(compress_layout(&best).per_warp) * t.warps_per_block >
+          static_cast<int64_t>(compress_layout(&best, glz::kMatchExact).per_warp) * t.warps_per_block >
               ctx->smem_optin)
         continue;  // this shape does not fit a block
       run(t);
