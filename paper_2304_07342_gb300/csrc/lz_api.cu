@@ -27,11 +27,11 @@ cudaError_t launch_compress_batch(const CompressArgs &A, const BufDesc *empties,
 cudaError_t launch_decompress_batch(DecompressBatchArgs B, int block, cudaStream_t stream);
 cudaError_t launch_stitch(const StitchArgs &A, int sms, cudaStream_t stream);
 cudaError_t launch_huff_compress(const uint8_t *in, uint64_t n, uint8_t *out, uint64_t out_cap,
-                                 unsigned long long *out_bytes, unsigned long long *hist,
-                                 uint32_t *book, uint32_t *err, int sms, cudaStream_t st);
+                                 unsigned long long *out_bytes, uint8_t *scratch, uint32_t *err,
+                                 int sms, cudaStream_t st);
 cudaError_t launch_huff_decompress(const uint8_t *in, uint64_t in_bytes, uint8_t *out,
                                    uint64_t out_cap, unsigned long long *out_bytes,
-                                   uint32_t *err, int sms, cudaStream_t st);
+                                   uint32_t *err, cudaStream_t st);
 uint64_t huff_layout_bits_at(uint64_t n);
 
 // Gather the 32-byte headers of n streams into one device array.
@@ -1540,12 +1540,10 @@ lz_status lz_huff_compress(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, void
   if (cudaSetDevice(ctx->device) != cudaSuccess) return LZ_ERR_CUDA;
   lz_status s = reserve_scratch(ctx, 4096);
   if (s != LZ_OK) return s;
-  auto *hist = static_cast<unsigned long long *>(ctx->scratch);
-  auto *book = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(ctx->scratch) + 2048);
   return cuda_status(glz::launch_huff_compress(
       static_cast<const uint8_t *>(d_in), n_bytes, static_cast<uint8_t *>(d_out), out_cap,
-      reinterpret_cast<unsigned long long *>(d_out_bytes), hist, book, ctx->d_err, ctx->sms,
-      reinterpret_cast<cudaStream_t>(stream)));
+      reinterpret_cast<unsigned long long *>(d_out_bytes), static_cast<uint8_t *>(ctx->scratch),
+      ctx->d_err, ctx->sms, reinterpret_cast<cudaStream_t>(stream)));
 }
 
 lz_status lz_huff_decompressed_size(const void *d_in, uint64_t in_bytes, uint64_t *h_n,
@@ -1578,7 +1576,7 @@ lz_status lz_huff_decompress(lz_ctx *ctx, const void *d_in, uint64_t in_bytes, v
   if (cudaSetDevice(ctx->device) != cudaSuccess) return LZ_ERR_CUDA;
   return cuda_status(glz::launch_huff_decompress(
       static_cast<const uint8_t *>(d_in), in_bytes, static_cast<uint8_t *>(d_out), out_cap,
-      reinterpret_cast<unsigned long long *>(d_out_bytes), ctx->d_err, ctx->sms,
+      reinterpret_cast<unsigned long long *>(d_out_bytes), ctx->d_err,
       reinterpret_cast<cudaStream_t>(stream)));
 }
 
