@@ -11,19 +11,18 @@
 //     with a TMA bulk copy; a chunk without pointers (or a stored chunk of
 //     stream version 2) is copied straight out with 16-byte stores;
 //   * otherwise the chunk is decoded into a shared-memory image of its
-//     output in two phases.  Phase 1 takes the tokens 32 at a time (lane =
-//     token): the flag word gives each token's payload offset by popcount,
-//     a shuffle scan of token lengths gives its output position; a literal
-//     writes its symbol there, a pointer writes (offset - 1) into the slot
-//     of its first symbol, and both mark their first position (one byte
-//     per position: literal or pointer start).  Phase 2 takes the output
-//     positions 32 at a time (lane = position): the owning token is the
-//     last marked position at or before the position (a ballot and a bit
-//     scan; a token that began in an earlier round is carried in
-//     registers), a position
-//     inside a pointer copies from position - offset, and sources inside
-//     the same 32 positions are resolved by pointer jumping over the lanes;
-//     earlier positions are final, later rounds read them;
+//     output in two phases, four tokens or positions per lane.  Phase 1
+//     takes 128 tokens a round: flag bits give each token's payload offset by
+//     popcount, a shuffle scan of the lanes' lengths its output position; a
+//     literal writes its symbol there, a pointer writes (offset - 1) into the
+//     slot of its first symbol, and both mark their first position (one byte
+//     per position: literal or pointer start).  Phase 2 takes 128 output
+//     positions a round: the owning token is the last marked position at or
+//     before the position (in the lane, in the lanes before it by a vote, or
+//     carried from the round before), a position inside a pointer copies from
+//     position - offset, and sources inside the round that are pointer
+//     symbols themselves are followed back through the round's offsets in
+//     shared memory; earlier positions are final, later rounds read them;
 //   * the image is copied out with 16-byte stores.
 // Pointers never reach before their own chunk, so chunks are independent
 // (section 3.3.1).  When the slice cannot hold the output image and the
@@ -191,6 +190,7 @@ __device__ __forceinline__ void copy_s2g(uint8_t *dst, const uint8_t *src,
 struct Slice {
   uint64_t *bar;
   uint8_t *marks;           // per position: 0 inside a token, 1 literal start, 2 pointer start
+  uint16_t *dist;           // per position of a round: how far back its source lies
   uint8_t *hi;              // high bytes of (offset - 1), or nullptr
   uint8_t *fl;              // a copy of the record's flag bytes
   uint8_t *io;              // output image + staged record, or nullptr (decode
@@ -203,6 +203,7 @@ __device__ __forceinline__ Slice make_slice(uint8_t *ws, const DecodeLayout &L, 
   Slice sl;
   sl.bar = reinterpret_cast<uint64_t *>(ws);
   sl.marks = ws + L.marks_off;
+  sl.dist = reinterpret_cast<uint16_t *>(ws + L.dist_off);
   sl.hi = hi ? ws + L.hi_off : nullptr;
   sl.fl = ws + L.flags_off;
   sl.io = L.staged ? ws + L.io_off : nullptr;
@@ -213,189 +214,280 @@ __device__ __forceinline__ Slice make_slice(uint8_t *ws, const DecodeLayout &L, 
   return sl;
 }
 
-// Flag word g of a record (tokens 32g .. 32g+31; bits of tokens past ntok
-// cleared).  STAGED: the flags are in shared memory, where a word may be
-// read past the flag bytes.
-template <bool STAGED>
-__device__ __forceinline__ uint32_t flag_word(const uint8_t *flags, uint32_t g, uint32_t ntok,
-                                              uint32_t fb) {
-  uint32_t fw;
-  if constexpr (STAGED) {
-    fw = ld_u32_any(flags + 4 * g);
+// Symbols per lane and round of the two phases: a lane takes four consecutive
+// tokens (phase 1) or positions (phase 2), so that votes, scans and the carry
+// from lane to lane are paid once per 128 instead of once per 32, and slots,
+// marks and payload move as words of four.  With one token or position per
+// lane the quantization codes took 8.0 K warp instructions per 4 KiB chunk
+// (issue-bound, 0.531 ms for 256 MiB).
+constexpr uint32_t kPer = 4, kRound = 32 * kPer;
+
+// The slots of positions j .. j + 3 (j a multiple of 4) of an output image.
+template <int S>
+__device__ __forceinline__ void ld_slots(const uint8_t *o, uint32_t j, uint32_t (&v)[kPer]) {
+  if constexpr (S == 1) {
+    const uint32_t w = *reinterpret_cast<const uint32_t *>(o + j);
+    v[0] = w & 0xFFu;
+    v[1] = (w >> 8) & 0xFFu;
+    v[2] = (w >> 16) & 0xFFu;
+    v[3] = w >> 24;
+  } else if constexpr (S == 2) {
+    const uint2 w = *reinterpret_cast<const uint2 *>(o + 2 * j);
+    v[0] = w.x & 0xFFFFu;
+    v[1] = w.x >> 16;
+    v[2] = w.y & 0xFFFFu;
+    v[3] = w.y >> 16;
   } else {
-    fw = 0;
-    for (uint32_t i = 0; i < 4; ++i)
-      if (4 * g + i < fb) fw |= static_cast<uint32_t>(flags[4 * g + i]) << (8 * i);
+    const uint4 w = *reinterpret_cast<const uint4 *>(o + 4 * j);
+    v[0] = w.x;
+    v[1] = w.y;
+    v[2] = w.z;
+    v[3] = w.w;
   }
-  const uint32_t left = ntok - 32 * g;
-  return left >= 32 ? fw : fw & ((1u << left) - 1u);
+}
+
+template <int S>
+__device__ __forceinline__ void st_slots(uint8_t *o, uint32_t j, const uint32_t (&v)[kPer]) {
+  if constexpr (S == 1) {
+    *reinterpret_cast<uint32_t *>(o + j) =
+        __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
+  } else if constexpr (S == 2) {
+    *reinterpret_cast<uint2 *>(o + 2 * j) =
+        make_uint2(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410));
+  } else {
+    *reinterpret_cast<uint4 *>(o + 4 * j) = make_uint4(v[0], v[1], v[2], v[3]);
+  }
 }
 
 // Phases 1 and 2 for a chunk of k symbols with ntok tokens whose payload
 // holds pay_tok bytes of tokens: the symbols are written into `ob` (the
-// output image, or the output itself).  STAGED: the record is in shared
-// memory (words may be read up to 3 bytes past it).  False when the tokens
-// are inconsistent (corrupt stream); nothing outside the chunk's output and
-// the slice is written either way.
+// output image, or the output itself).  The flag bytes are in sl.fl, bits
+// past ntok cleared up to the next multiple of 128.  STAGED: the record is in
+// shared memory (words may be read up to 12 bytes past it) and `ob` is the
+// image.  False when the tokens are inconsistent (corrupt stream); nothing
+// outside the chunk's output and the slice is written either way.
 // SAME: a pointer's payload is S bytes like a literal's (1 + offB == S), so
 // token t's payload starts at S * t without counting the pointers before it.
 template <int S, bool STAGED, bool SAME = false>
-__device__ __forceinline__ bool decode_tokens(const Header &h, const uint8_t *flags,
-                                              const uint8_t *payload, uint32_t ntok,
-                                              uint32_t pay_tok, uint32_t k, uint8_t *ob,
-                                              bool aligned, const Slice &sl, uint32_t lane) {
+__device__ __forceinline__ bool decode_tokens(const Header &h, const uint8_t *payload,
+                                              uint32_t ntok, uint32_t pay_tok, uint32_t k,
+                                              uint8_t *ob, bool aligned, const Slice &sl,
+                                              uint32_t lane) {
   const uint32_t tsz = 1u + h.offB;
   const uint32_t offmask = h.offB == 2 ? 0xFFFFu : 0xFFu;
   const uint32_t lt = lanemask_lt(lane);
-  const uint32_t fb = (ntok + 7) / 8;
   uint8_t *marks = sl.marks;
+  const uint32_t *fw = reinterpret_cast<const uint32_t *>(sl.fl);
   {
     uint4 *m16 = reinterpret_cast<uint4 *>(marks);
-    const uint32_t n16 = ((k + 31) & ~31u) / 16;
+    const uint32_t n16 = ((k + kRound - 1) & ~(kRound - 1)) / 16;
     for (uint32_t i = lane; i < n16; i += 32) m16[i] = make_uint4(0, 0, 0, 0);
   }
   __syncwarp();
 
-  // Phase 1: tokens (lane = token), two groups of 32 per step.  The flag
-  // words are read 32 at a time (lane = group); a scan of their popcounts
-  // gives every group the pointers before it, so each token's payload
-  // offset follows without a running sum: S bytes per literal and 1 + offB
-  // per pointer before it.  The payload must hold exactly the flagged
-  // tokens, checked before any token is read.
-  const uint32_t ngroups = (ntok + 31) / 32;
+  // Phase 1: tokens.  A lane's four flag bits and, unless SAME, the pointers
+  // before them in the round (popcounts of the round's four flag words) give
+  // its tokens' payload offsets: S bytes per literal and 1 + offB per pointer
+  // before it.  One scan of the lanes' lengths gives the output positions.
+  // The payload must hold exactly the flagged tokens, checked before any
+  // token is read.
   uint32_t np = 0;
-  for (uint32_t g = lane; g < ngroups; g += 32)
-    np += __popc(flag_word<STAGED>(flags, g, ntok, fb));
+  for (uint32_t g = lane; g < (ntok + 31) / 32; g += 32) np += __popc(fw[g]);
   np = __reduce_add_sync(kFull, np);
   if (S * (ntok - np) + tsz * np != pay_tok) return false;
-  auto put = [&](uint32_t st, bool m, uint32_t off, uint32_t w) {
-    if (!GLZ_OK(st < k && st < sl.mark_bytes)) return;
-    marks[st] = m ? 2 : 1;
-    st_slot<S>(ob, st, m ? off - 1u : w, aligned);
-    if (S == 1 && sl.hi && m) sl.hi[st] = static_cast<uint8_t>((off - 1u) >> 8);
-  };
-  uint32_t pos = 0, pdone = 0;  // symbols produced; pointers in earlier blocks of groups
-  for (uint32_t g0 = 0; g0 < ngroups; g0 += 32) {
-    const uint32_t fwr = g0 + lane < ngroups ? flag_word<STAGED>(flags, g0 + lane, ntok, fb) : 0u;
-    uint32_t pb = 0;  // pointers before group g0 + lane (not needed when SAME)
-    if constexpr (!SAME) {
-      const uint32_t cnt = __popc(fwr);
-      uint32_t incl = cnt;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= static_cast<uint32_t>(o)) incl += y;
-      }
-      pb = pdone + incl - cnt;
-      pdone += __shfl_sync(kFull, incl, 31);
-    }
-    const uint32_t nblk = min(32u, ngroups - g0);
-    for (uint32_t i = 0; i < nblk; i += 2) {
-      const bool hasB = i + 1 < nblk;
-      const uint32_t fwA = __shfl_sync(kFull, fwr, i);
-      const uint32_t fwB = __shfl_sync(kFull, fwr, (i + 1) & 31u);
-      const uint32_t tA = (g0 + i) * 32 + lane, tB = tA + 32;
-      const bool vA = tA < ntok, vB = hasB && tB < ntok;
-      const bool mA = (fwA >> lane) & 1u, mB = hasB && ((fwB >> lane) & 1u);
-      uint32_t oA = S * tA, oB = S * tB;
-      if constexpr (!SAME) {
-        const uint32_t pbA = __shfl_sync(kFull, pb, i), pbB = __shfl_sync(kFull, pb, (i + 1) & 31u);
-        const uint32_t nbA = pbA + __popc(fwA & lt), nbB = pbB + __popc(fwB & lt);
-        oA = S * (tA - nbA) + tsz * nbA;
-        oB = S * (tB - nbB) + tsz * nbB;
-      }
-      uint32_t wA = 0, wB = 0;
-      if constexpr (STAGED) {
-        if (vA && GLZ_OK(oA < pay_tok)) wA = ld_u32_any(payload + oA);
-        if (vB && GLZ_OK(oB < pay_tok)) wB = ld_u32_any(payload + oB);
+  uint32_t pos = 0, pdone = 0;  // symbols produced; pointers in earlier rounds
+#pragma unroll 1
+  for (uint32_t t0 = 0; t0 < ntok; t0 += kRound) {
+    const uint32_t t = t0 + kPer * lane;
+    const uint32_t nv = t < ntok ? min(kPer, ntok - t) : 0u;
+    const uint32_t own = fw[t0 / 32 + (lane >> 3)], at = kPer * (lane & 7u);
+    const uint32_t f = own >> at;
+    uint32_t w[kPer];
+    if constexpr (SAME && STAGED) {
+      if (nv && GLZ_OK(S * t < pay_tok)) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(payload + S * t);
+        const uint32_t *p = reinterpret_cast<const uint32_t *>(a & ~static_cast<uintptr_t>(3));
+        const uint32_t sh = 8u * static_cast<uint32_t>(a & 3u);  // 0 or 16
+        const uint32_t x = p[0], y = p[1], z = p[2];
+        const uint32_t lo = __funnelshift_r(x, y, sh), hi = __funnelshift_r(y, z, sh);
+        w[0] = lo & 0xFFFFu;
+        w[1] = lo >> 16;
+        w[2] = hi & 0xFFFFu;
+        w[3] = hi >> 16;
       } else {
-        if (vA) wA = static_cast<uint32_t>(ld_le(payload + oA, mA ? tsz : S));
-        if (vB) wB = static_cast<uint32_t>(ld_le(payload + oB, mB ? tsz : S));
+        w[0] = w[1] = w[2] = w[3] = 0;
       }
-      const uint32_t lenA = mA ? (wA & 0xFFu) : (vA ? 1u : 0u);
-      const uint32_t lenB = mB ? (wB & 0xFFu) : (vB ? 1u : 0u);
-      const uint32_t offA = mA ? ((wA >> 8) & offmask) + 1u : 0u;
-      const uint32_t offB = mB ? ((wB >> 8) & offmask) + 1u : 0u;
-      // inclusive scans of both groups' token lengths in one: A in the low
-      // and B in the high 16 bits (a group's lengths sum to at most
-      // 32 x 255, so the halves never carry into each other)
-      uint32_t x = lenA | (lenB << 16);
+    } else {
+      const uint4 all = *reinterpret_cast<const uint4 *>(fw + t0 / 32);
+      const uint32_t c0 = __popc(all.x), c1 = c0 + __popc(all.y), c2 = c1 + __popc(all.z);
+      const uint32_t g = lane >> 3;
+      uint32_t before = g == 0 ? 0u : g == 1 ? c0 : g == 2 ? c1 : c2;
+      before += pdone + __popc(own & ((1u << at) - 1u));
+      pdone += c2 + __popc(all.w);
+      uint32_t o = S * (t - before) + tsz * before;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, x, o);
-        if (lane >= static_cast<uint32_t>(o)) x += y;
+      for (uint32_t i = 0; i < kPer; ++i) {
+        const bool m = (f >> i) & 1u;
+        w[i] = 0;
+        if (i < nv && GLZ_OK(o < pay_tok)) {
+          if constexpr (STAGED) w[i] = ld_u32_any(payload + o);
+          else w[i] = static_cast<uint32_t>(ld_le(payload + o, m ? tsz : S));
+        }
+        o += m ? tsz : S;
       }
-      const uint32_t gl2 = __shfl_sync(kFull, x, 31);
-      const uint32_t xA = x & 0xFFFFu, xB = x >> 16;
-      const uint32_t glA = gl2 & 0xFFFFu, glB = gl2 >> 16;
-      const uint32_t sA = pos + xA - lenA, sB = pos + glA + xB - lenB;
-      // a pointer needs 1 <= length <= offset (any length <= 255 in overlap
-      // mode) and offset <= min(W, its start): its source lies in the chunk
-      const uint32_t capA = h.overlap ? 256u : offA, capB = h.overlap ? 256u : offB;
-      const bool bad = (mA && !(lenA - 1u < capA && offA <= min(h.W, sA))) ||
-                       (mB && !(lenB - 1u < capB && offB <= min(h.W, sB)));
-      if (__any_sync(kFull, bad) || pos + glA + glB > k) return false;
-      pos += glA + glB;
-      if (vA) put(sA, mA, offA, wA);
-      if (vB) put(sB, mB, offB, wB);
+    }
+    uint32_t len[kPer], off[kPer], sum = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      const bool m = (f >> i) & 1u;
+      len[i] = m ? w[i] & 0xFFu : (i < nv ? 1u : 0u);
+      off[i] = ((w[i] >> 8) & offmask) + 1u;
+      sum += len[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= static_cast<uint32_t>(o)) incl += y;
+    }
+    uint32_t st = pos + incl - sum;
+    pos += __shfl_sync(kFull, incl, 31);
+    // a pointer needs 1 <= length <= offset (any length <= 255 in overlap
+    // mode) and offset <= min(W, its start): its source lies in the chunk
+    bool bad = pos > k;
+    uint32_t start[kPer];
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      start[i] = st;
+      const uint32_t cap = h.overlap ? 256u : off[i];
+      bad |= ((f >> i) & 1u) && !(len[i] - 1u < cap && off[i] <= min(h.W, st));
+      st += len[i];
+    }
+    if (__any_sync(kFull, bad)) return false;
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      if (i >= nv || !GLZ_OK(start[i] < k && start[i] < sl.mark_bytes)) continue;
+      const bool m = (f >> i) & 1u;
+      marks[start[i]] = m ? 2 : 1;
+      st_slot<S>(ob, start[i], m ? off[i] - 1u : w[i], aligned);
+      if (S == 1 && sl.hi && m) sl.hi[start[i]] = static_cast<uint8_t>((off[i] - 1u) >> 8);
     }
   }
   if (pos != k) return false;
   __syncwarp();
 
-  // Phase 2: positions, 32 at a time (lane = position)
-  const uint32_t le = lt | (1u << lane);
-  uint32_t carry = 0;  // offset of the pointer owning the previous round's last position (0: literal)
-  for (uint32_t r0 = 0; r0 < k; r0 += 32) {
-    const uint32_t j = r0 + lane;
-    const bool act = j < k;
-    const uint32_t mk = marks[j];  // zero past k
-    const uint32_t sw = __ballot_sync(kFull, mk != 0);
-    // the offset of the pointer starting here (its slot holds offset - 1);
-    // 0 at a literal's start
-    uint32_t so = 0;
-    if constexpr (S == 1) {  // (a byte load costs less than the branch around it)
-      uint32_t raw = act ? ld_slot<S>(ob, j, aligned) : 0u;
-      if (sl.hi && act) raw |= static_cast<uint32_t>(sl.hi[j]) << 8;
-      so = mk == 2 ? raw + 1u : 0u;
-    } else if (mk == 2) {
-      so = ld_slot<S>(ob, j, aligned) + 1u;
+  // Phase 2: positions.  A position's offset is that of the token it lies in
+  // (0: a literal), carried from lane to lane by one vote and one shuffle per
+  // round.  Offsets of the round go to sl.dist; a source inside the round
+  // that is itself a pointer symbol is followed back through them until it is
+  // a literal of the round or lies before it (2 to 3 turns on codes with 50
+  // to 80 % pointer symbols).
+  uint32_t carry = 0;  // offset owning the previous round's last position
+#pragma unroll 1
+  for (uint32_t r0 = 0; r0 < k; r0 += kRound) {
+    const uint32_t x0 = kPer * lane, j = r0 + x0;
+    const uint32_t nv = j < k ? min(kPer, k - j) : 0u;
+    const uint32_t mk = *reinterpret_cast<const uint32_t *>(marks + j);  // zero past k
+    uint32_t v[kPer] = {0, 0, 0, 0};
+    if constexpr (STAGED) {
+      if (nv) ld_slots<S>(ob, j, v);
+    } else {
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i)
+        if (i < nv) v[i] = ld_slot<S>(ob, j + i, aligned);
     }
-    const uint32_t mb = sw & le;
-    const uint32_t ol = (31u - __clz(mb)) & 31u;  // owner's lane when mb != 0
-    const uint32_t oso = __shfl_sync(kFull, so, ol);
-    const uint32_t own = mb ? oso : carry;
+    uint32_t s[kPer];  // offset of the token starting here (0: literal)
+    if (S == 1 && sl.hi) {
+      const uint32_t hw = nv ? *reinterpret_cast<const uint32_t *>(sl.hi + j) : 0u;
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) s[i] = (v[i] | (((hw >> (8 * i)) & 0xFFu) << 8)) + 1u;
+    } else {
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) s[i] = v[i] + 1u;
+    }
+    uint32_t last = 0;  // that of the lane's last start
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      const uint32_t b = (mk >> (8 * i)) & 0xFFu;
+      s[i] = b == 2 ? s[i] : 0u;
+      last = b ? s[i] : last;
+    }
+    const uint32_t starts = __ballot_sync(kFull, mk != 0);
+    const uint32_t prev = starts & lt;
+    const uint32_t from_lane = __shfl_sync(kFull, last, (31u - __clz(prev)) & 31u);
+    uint32_t own = prev ? from_lane : carry;
+    uint32_t off[kPer], f[kPer];
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      own = (mk >> (8 * i)) & 0xFFu ? s[i] : own;
+      off[i] = i < nv ? own : 0u;
+      f[i] = j + i - off[i];
+    }
     carry = __shfl_sync(kFull, own, 31);
-    const bool ptr = act && own != 0;
-    uint32_t f = ptr ? j - own : j;
-    // sources inside this round that are pointer symbols themselves are not
-    // final yet: jump (f <- the source's source, all lanes at once) until
-    // every source is a literal of the round or lies before it (chains
-    // shrink, so at most 5 turns)
-    const uint32_t pm = __ballot_sync(kFull, ptr);
-    auto pending = [&](uint32_t x) { return x >= r0 && ((pm >> (x - r0)) & 1u); };
-    while (__any_sync(kFull, pending(f))) f = __shfl_sync(kFull, f, pending(f) ? f - r0 : lane);
-    if (ptr && GLZ_OK(f < j)) st_slot<S>(ob, j, ld_slot<S>(ob, f, aligned), aligned);
+    uint2 *mine = reinterpret_cast<uint2 *>(sl.dist + x0);
+    *mine = make_uint2(__byte_perm(off[0], off[1], 0x5410), __byte_perm(off[2], off[3], 0x5410));
+    __syncwarp();
+    // one turn: every source in the round moves to its own source
+    auto turn = [&]() -> bool {
+      uint32_t moved = 0;
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) {
+        uint32_t d = 0;
+        if (off[i] && f[i] >= r0) d = sl.dist[f[i] - r0];
+        f[i] -= d;
+        moved |= d;
+      }
+      return moved != 0;
+    };
+    bool again = true;
+    for (uint32_t n = 0; again && n < 4; ++n) again = turn();
+    // long chains (matches that overlap their output): the distances already
+    // followed replace the offsets, which doubles the reach of a turn.  A
+    // lane may see another's old or new distance; both lead back along the
+    // same chain.
+    while (__any_sync(kFull, again)) {
+      uint32_t d[kPer];
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i) d[i] = j + i - f[i];
+      *mine = make_uint2(__byte_perm(d[0], d[1], 0x5410), __byte_perm(d[2], d[3], 0x5410));
+      __syncwarp();
+      again = turn();
+    }
+    uint32_t any = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < kPer; ++i) {
+      any |= off[i];
+      if (off[i] && GLZ_OK(f[i] < j + i)) v[i] = ld_slot<S>(ob, f[i], aligned);
+    }
+    // (a literal's slot is written again with its own value: other lanes of
+    // the round may be reading it)
+    if constexpr (STAGED) {
+      if (any) st_slots<S>(ob, j, v);
+    } else {
+#pragma unroll
+      for (uint32_t i = 0; i < kPer; ++i)
+        if (off[i]) st_slot<S>(ob, j + i, v[i], aligned);
+    }
     __syncwarp();
   }
   return true;
 }
 
 template <bool STAGED>
-__device__ __forceinline__ bool decode_tokens_s(const Header &h, const uint8_t *flags,
-                                                const uint8_t *payload, uint32_t ntok,
+__device__ __forceinline__ bool decode_tokens_s(const Header &h, const uint8_t *payload,
+                                                uint32_t ntok,
                                                 uint32_t pay_tok, uint32_t k, uint8_t *ob,
                                                 bool aligned, const Slice &sl, uint32_t lane) {
   switch (h.S) {
     case 1:
-      return decode_tokens<1, STAGED>(h, flags, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
+      return decode_tokens<1, STAGED>(h, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
     case 2:
       if (h.offB == 1)  // a pointer (length, offset - 1) is two bytes, as a symbol
-        return decode_tokens<2, STAGED, true>(h, flags, payload, ntok, pay_tok, k, ob, aligned, sl,
+        return decode_tokens<2, STAGED, true>(h, payload, ntok, pay_tok, k, ob, aligned, sl,
                                               lane);
-      return decode_tokens<2, STAGED>(h, flags, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
+      return decode_tokens<2, STAGED>(h, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
     default:
-      return decode_tokens<4, STAGED>(h, flags, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
+      return decode_tokens<4, STAGED>(h, payload, ntok, pay_tok, k, ob, aligned, sl, lane);
   }
 }
 
@@ -475,16 +567,22 @@ __device__ __forceinline__ bool decode_chunk(const DecompressArgs &A, const Head
   // the tail bytes, read before the output image may grow over the record
   const uint8_t tb = lane < tail ? payload[pay_tok + lane] : 0;
   bool ok;
+  // the flag bytes are copied out first (the output image grows from the
+  // start of the io area towards the record's flags), the bits past the last
+  // token cleared up to a round of the token phase
+  const uint32_t fpad = (static_cast<uint32_t>(fb) + 15u) & ~15u;
+  if (!GLZ_OK(fpad <= sl.flag_bytes)) return true;
+  for (uint32_t i = lane; i < fpad; i += 32) {
+    uint32_t v = i < fb ? flags[i] : 0u;
+    if (i + 1 == fb && (ntok & 7u)) v &= (1u << (ntok & 7u)) - 1u;
+    sl.fl[i] = static_cast<uint8_t>(v);
+  }
+  __syncwarp();
   if (sl.io) {
-    // the flag bytes are copied out first: the output image grows from the
-    // start of the io area towards the record's flags
-    if (!GLZ_OK(fb + 8 <= sl.flag_bytes)) return true;
-    for (uint32_t i = lane; i < fb; i += 32) sl.fl[i] = flags[i];
-    __syncwarp();
-    ok = decode_tokens_s<true>(h, sl.fl, payload, ntok, pay_tok, k, sl.io, true, sl, lane);
+    ok = decode_tokens_s<true>(h, payload, ntok, pay_tok, k, sl.io, true, sl, lane);
   } else {
     const bool aligned = A.out_aligned != 0 && (h.C % 4) == 0;
-    ok = decode_tokens_s<false>(h, flags, payload, ntok, pay_tok, k, dst, aligned, sl, lane);
+    ok = decode_tokens_s<false>(h, payload, ntok, pay_tok, k, dst, aligned, sl, lane);
   }
   if (!ok) {
     if (lane == 0) atomicOr(A.err, kErrCorrupt);

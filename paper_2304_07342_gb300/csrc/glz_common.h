@@ -139,7 +139,7 @@ struct DecItem {
 // Per-warp shared-memory slice of the decoder (byte offsets, 16-byte
 // aligned): an mbarrier, one mark byte per position of the chunk (0 inside
 // a token, 1 where a literal starts, 2 where a pointer starts), a copy of
-// the record's flag bytes, the high bytes of (offset - 1) when one-byte
+// the record's flag bytes, a round's source distances, the high bytes of (offset - 1) when one-byte
 // symbols carry two-byte offsets, then -- when they fit -- the io area:
 // the chunk's output image from its start, with the record staged at its
 // end.  When no pointer takes more payload bytes than the symbols it
@@ -149,10 +149,11 @@ struct DecItem {
 // by side.  Without the io area (`staged` false) a warp decodes straight
 // into the output buffer and reads the record in place.
 struct DecodeLayout {
-  uint32_t marks_off;  // mark bytes, a multiple of 32
+  uint32_t marks_off;  // mark bytes, a multiple of 128 (a round of positions)
   uint32_t mark_bytes;
   uint32_t flags_off;  // flag bytes of one record (+ 16 slack)
   uint32_t flag_bytes;
+  uint32_t dist_off;   // 128 source distances (u16), one round of positions
   uint32_t hi_off;     // k bytes (one-byte symbols, two-byte offsets) or none
   uint32_t io_off;     // output image + staged record
   uint32_t io_bytes;
@@ -181,11 +182,13 @@ __host__ __device__ inline DecodeLayout decode_layout(uint64_t kmax, uint64_t cm
   DecodeLayout L{};
   uint64_t at = 16;  // mbarrier
   L.marks_off = static_cast<uint32_t>(at);
-  L.mark_bytes = static_cast<uint32_t>((kmax + 31) & ~31ull);
+  L.mark_bytes = static_cast<uint32_t>((kmax + 127) & ~127ull);
   at += L.mark_bytes;
   L.flags_off = static_cast<uint32_t>(at);
   L.flag_bytes = static_cast<uint32_t>(((kmax + 7) / 8 + 15) & ~15ull) + 16;
   at += L.flag_bytes;
+  L.dist_off = static_cast<uint32_t>(at);
+  at += 256;
   L.hi_off = static_cast<uint32_t>(at);
   if (hi) at += (kmax + 15) & ~15ull;
   const uint64_t base = at;
