@@ -1,8 +1,15 @@
-// compress_batch.cu -- one persistent launch over the chunks of many buffers
-// (each with its own parameters), plus the headers of empty buffers.
-#include "compress_batch_launch.cuh"
+// compress_batch.cu -- the launches of a compression batch: the headers of
+// empty buffers and one launch per class of buffers.
+#include "compress_impl.cuh"
 
 namespace glz {
+
+cudaError_t launch_batch_s1(const CompressArgs &A, uint32_t nj, bool mask, int block,
+                            unsigned grid, cudaStream_t stream);
+cudaError_t launch_batch_s2(const CompressArgs &A, uint32_t nj, bool mask, int block,
+                            unsigned grid, cudaStream_t stream);
+cudaError_t launch_batch_s4(const CompressArgs &A, uint32_t nj, bool mask, int block,
+                            unsigned grid, cudaStream_t stream);
 
 // Empty buffers: their stream is the header alone.
 __global__ void batch_empty_headers(const BufDesc *empties, uint32_t n) {
@@ -15,21 +22,17 @@ __global__ void batch_empty_headers(const BufDesc *empties, uint32_t n) {
   }
 }
 
-cudaError_t launch_compress_batch(const CompressArgs &A, const BufDesc *empties,
-                                  uint32_t n_empty, uint32_t nj, int block, unsigned grid,
-                                  cudaStream_t stream) {
-  if (n_empty) {
-    batch_empty_headers<<<(n_empty + 7) / 8, 256, 0, stream>>>(empties, n_empty);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  if (A.total_chunks == 0) return cudaSuccess;
-  switch (nj) {
-    case 1:
-    case 2:
-    case 4: return launch_batch_nj<4>(A, block, grid, stream);
-    case 8: return launch_batch_nj<8>(A, block, grid, stream);
-    default: return launch_batch_wide(A, nj, block, grid, stream);
+cudaError_t launch_batch_empties(const BufDesc *empties, uint32_t n, cudaStream_t stream) {
+  batch_empty_headers<<<(n + 7) / 8, 256, 0, stream>>>(empties, n);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_batch_class(const CompressArgs &A, uint32_t S, uint32_t nj, bool mask,
+                               int block, unsigned grid, cudaStream_t stream) {
+  switch (S) {
+    case 1: return launch_batch_s1(A, nj, mask, block, grid, stream);
+    case 2: return launch_batch_s2(A, nj, mask, block, grid, stream);
+    default: return launch_batch_s4(A, nj, mask, block, grid, stream);
   }
 }
 

@@ -1211,53 +1211,30 @@ __device__ __forceinline__ uint32_t find_item(const CompressArgs &A, uint64_t g,
   return lo;
 }
 
-// A chunk of a batch, by its buffer's symbol size.  (Out of line: one copy
-// of each variant, whatever the number of kernels.)
-template <int S, int NJ, bool WIDE, bool MASK>
-__device__ __noinline__ bool batch_chunk(const CompressArgs &A, const BufDesc &item_desc,
-                                         uint32_t item, uint32_t c, WarpState &W, uint32_t lane) {
-  const BufDesc B = item_desc;
-  return compress_chunk<S, NJ, WIDE, MASK>(A, B, item, c, W, lane);
-}
-
-template <int NJ, bool WIDE, bool MASK>
-__device__ __forceinline__ bool compress_item(const CompressArgs &A, const BufDesc &B,
-                                              uint32_t item, uint32_t c, WarpState &W,
-                                              uint32_t lane) {
-  switch (B.S) {
-    case 1: return batch_chunk<1, NJ, WIDE, MASK>(A, B, item, c, W, lane);
-    case 2: return batch_chunk<2, NJ, WIDE, MASK>(A, B, item, c, W, lane);
-    default: return batch_chunk<4, NJ, WIDE, MASK>(A, B, item, c, W, lane);
-  }
-}
-
-// Batch: work items are the chunks of all buffers in order; each buffer
-// carries its own parameters, so the symbol size is dispatched per chunk.
-template <int NJ>
-__global__ void __launch_bounds__(256, min_blocks(NJ, true))
-    compress_batch_kernel(const __grid_constant__ CompressArgs A) {
+// Batch: work items are the chunks of all buffers of one class (one symbol
+// size, parse and range of windows) in order; each buffer carries its own
+// parameters, kept in shared memory while one of its chunks is compressed.
+template <int S, int NJ, bool MASK>
+__global__ void __launch_bounds__(256, min_blocks(NJ, MASK))
+    compress_batch_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
+  __shared__ BufDesc descs[8];
   const uint32_t lane = threadIdx.x & 31;
+  BufDesc &B = descs[threadIdx.x >> 5];
   WarpState W;
   init_warp_state(A, smem, W, lane);
   while (true) {
     const uint32_t g = take_ticket(A, lane);
     if (g >= A.total_chunks) break;
     const uint32_t item = find_item(A, g, lane);
-    const BufDesc B = A.items[item];
+    static_assert(sizeof(BufDesc) % 4 == 0 && sizeof(BufDesc) <= 128, "one word per lane");
+    if (lane < sizeof(BufDesc) / 4)
+      reinterpret_cast<uint32_t *>(&B)[lane] =
+          reinterpret_cast<const uint32_t *>(A.items + item)[lane];
+    __syncwarp();
     const uint32_t c = static_cast<uint32_t>(g - B.gbase);
-    bool ok;
-    if (mask_parse_takes(B.S, B.W, B.m, B.match)) {
-      // (an instance for each class of windows: a mask word costs every position)
-      if (NJ <= 4 || B.W <= 128) ok = compress_item<4, false, true>(A, B, item, c, W, lane);
-      else if (NJ <= 8 || B.W <= 256) ok = compress_item<8, false, true>(A, B, item, c, W, lane);
-      else ok = compress_item<16, false, true>(A, B, item, c, W, lane);
-    } else if (NJ <= 8 || B.W <= 256) {
-      ok = compress_item<(NJ < 8 ? NJ : 8), false, false>(A, B, item, c, W, lane);
-    } else {
-      ok = compress_item<NJ, true, false>(A, B, item, c, W, lane);
-    }
-    if (!ok) break;
+    if (!compress_chunk<S, NJ, (NJ > 8), MASK>(A, B, item, c, W, lane)) break;
+    __syncwarp();
   }
   drain_parked(A, W, true, lane);
   if (lane == 0) checked_fold(A.err);

@@ -21,9 +21,9 @@ cudaError_t launch_compress_s2(const CompressArgs &A, uint32_t nj, int block,
 cudaError_t launch_compress_s4(const CompressArgs &A, uint32_t nj, int block,
                                unsigned grid, cudaStream_t stream);
 cudaError_t launch_decompress(DecompressArgs A, int block, cudaStream_t stream);
-cudaError_t launch_compress_batch(const CompressArgs &A, const BufDesc *empties,
-                                  uint32_t n_empty, uint32_t nj, int block, unsigned grid,
-                                  cudaStream_t stream);
+cudaError_t launch_batch_empties(const BufDesc *empties, uint32_t n, cudaStream_t stream);
+cudaError_t launch_batch_class(const CompressArgs &A, uint32_t S, uint32_t nj, bool mask,
+                               int block, unsigned grid, cudaStream_t stream);
 cudaError_t launch_decompress_batch(DecompressBatchArgs B, int block, cudaStream_t stream);
 cudaError_t launch_stitch(const StitchArgs &A, int sms, cudaStream_t stream);
 cudaError_t launch_huff_compress(const uint8_t *in, uint64_t n, uint8_t *out, uint64_t out_cap,
@@ -953,9 +953,21 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
 enum BatchBuf { kBufScratch, kBufItems, kBufBases, kBufEmpties, kBufIns, kBufInBytes, kBufHdr,
                 kBufCount };
 
+constexpr int kBatchSides = 3;
+
 struct DevBuf {
   void *p = nullptr;
   size_t cap = 0;
+};
+
+// The buffers of a compression batch that one launch takes: one symbol size,
+// one parse (masks or chains) and one range of windows.
+struct BatchClass {
+  uint32_t S = 1, nj = 4;
+  bool mask = false;
+  int block = 32;
+  unsigned grid = 1;
+  glz::CompressArgs args{};
 };
 
 struct lz_batch {
@@ -968,12 +980,15 @@ struct lz_batch {
   cudaStream_t stream = nullptr;  // allocations and uploads are ordered on it
   DevBuf bufs[kBufCount];         // device allocations owned by the batch
   // compression
-  glz::CompressArgs cargs{};
+  std::vector<BatchClass> classes;  // most work first
   const glz::BufDesc *d_empty = nullptr;
-  uint32_t n_empty = 0, nj = 1;
-  int block = 32;
-  unsigned grid = 1;
+  uint32_t n_empty = 0;
   size_t clear_bytes = 0;
+  // launches of the classes after the first, forked from and joined to the
+  // caller's stream
+  cudaStream_t side[kBatchSides] = {};
+  cudaEvent_t fork = nullptr, join[kBatchSides] = {};
+  std::mutex run_mu;  // a run's fork and join use the batch's events
   void *scratch = nullptr;
   // decompression
   glz::DecompressBatchArgs dargs{};
@@ -1053,14 +1068,29 @@ glz::CompressSmem compress_layout_max(const std::vector<lz_params> &ps, uint32_t
   return sm;
 }
 
+void batch_streams_free(lz_batch *b) {
+  for (int i = 0; i < kBatchSides; ++i) {
+    if (b->join[i]) cudaEventDestroy(b->join[i]);
+    if (b->side[i]) cudaStreamDestroy(b->side[i]);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
+}
+
+// A compression batch is one launch per class of buffers (BatchClass), the
+// classes side by side on streams of the batch.  One launch over everything
+// sized every warp's slice and registers for the largest item: with 1-, 2-
+// and 4-byte requests 11 warps per SM, 34 % of issue slots used.
 lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_t n,
                                 lz_batch *b, uint32_t match, uint32_t version) {
-  const uint32_t warps_per_block = b->warps_per_block;
-  std::vector<glz::BufDesc> descs, empties;
-  std::vector<uint64_t> bases;
-  std::vector<lz_params> ps;
-  uint64_t total = 0, kmax = 1;
-  uint32_t nj = 1;
+  struct Group {
+    BatchClass cls;
+    std::vector<glz::BufDesc> descs;
+    std::vector<lz_params> ps;
+    uint64_t chunks = 0, bytes = 0;
+  };
+  std::vector<Group> groups;
+  std::vector<glz::BufDesc> empties;
+  uint64_t total = 0;
   for (uint32_t i = 0; i < n; ++i) {
     const lz_batch_item &it = items[i];
     const lz_params *p = &it.params;
@@ -1088,73 +1118,139 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
     d.nc = static_cast<uint32_t>(nc);
     d.in_aligned = (reinterpret_cast<uintptr_t>(it.d_in) % 16) == 0;
     d.records_at = records_at;
-    d.gbase = total;
     d.match = match;
     d.version = version;
     if (nc == 0) {
       empties.push_back(d);
       continue;
     }
-    descs.push_back(d);
-    bases.push_back(total);
     total += nc;
     if (total > kMaxLaunchChunks) return LZ_ERR_INVALID_ARG;
-    ps.push_back(*p);
-    kmax = std::max<uint64_t>(kmax, p->chunk_bytes / p->symbol_bytes);
-    uint32_t j = 1;
-    while (32 * j < p->window) j *= 2;
-    nj = std::max(nj, j);
+    const bool mask = glz::mask_parse_takes(d.S, d.W, d.m, match);
+    uint32_t nj = mask ? 4 : 8;
+    while (32 * nj < p->window) nj *= mask ? 2 : 4;
+    Group *g = nullptr;
+    for (Group &x : groups)
+      if (x.cls.S == d.S && x.cls.nj == nj && x.cls.mask == mask) g = &x;
+    if (!g) {
+      groups.emplace_back();
+      g = &groups.back();
+      g->cls.S = d.S;
+      g->cls.nj = nj;
+      g->cls.mask = mask;
+    }
+    d.gbase = g->chunks;
+    g->chunks += nc;
+    g->bytes += it.in_bytes;
+    g->descs.push_back(d);
+    g->ps.push_back(*p);
   }
-  glz::CompressSmem sm = ps.empty() ? glz::CompressSmem{} : compress_layout_max(ps, match);
-  if (!ps.empty() && static_cast<int64_t>(sm.per_warp) > ctx->smem_optin)
-    return LZ_ERR_INVALID_ARG;
-  int block = 32;
-  int64_t best_blocks = 1;
-  if (!ps.empty() && !block_shape(sm.per_warp, ctx->smem_per_sm, ctx->smem_reserved,
-                                  ctx->smem_optin, warps_per_block, &block, &best_blocks))
-    return LZ_ERR_INVALID_ARG;
-  const uint64_t wpb = block / 32;
-  uint64_t grid = std::max<uint64_t>(1, div_up(total, wpb));
-  if (grid > static_cast<uint64_t>(best_blocks) * ctx->sms) grid = best_blocks * ctx->sms;
-  uint64_t rb_max = 0;  // a parking slot holds any item's largest record
-  for (const lz_params &q : ps)
-    rb_max = std::max<uint64_t>(rb_max, record_bound(q.chunk_bytes / q.symbol_bytes,
-                                                     q.symbol_bytes, off_bytes(q.window),
-                                                     q.min_match) +
-                                            q.symbol_bytes);
-  const uint32_t slot_bytes = round16(rb_max + 16);
-  const size_t status_end = kScratchHead + 8ull * total;
-  const size_t park_at = (status_end + 255) & ~static_cast<size_t>(255);
-  const size_t scratch = park_at + static_cast<size_t>(slot_bytes) * kParkSlots * wpb * grid;
-  lz_status s = batch_alloc(b, kBufScratch, scratch, &b->scratch);
+  std::sort(groups.begin(), groups.end(),
+            [](const Group &x, const Group &y) { return x.bytes > y.bytes; });
+  // scratch: every class's work counter and look-back words, then the parking
+  // slots of every class
+  size_t clear = 0, park = 0;
+  std::vector<size_t> clear_at, park_at;
+  for (Group &g : groups) {
+    const glz::CompressSmem sm = compress_layout_max(g.ps, match);
+    if (static_cast<int64_t>(sm.per_warp) > ctx->smem_optin) return LZ_ERR_INVALID_ARG;
+    int64_t best_blocks = 1;
+    if (!block_shape(sm.per_warp, ctx->smem_per_sm, ctx->smem_reserved, ctx->smem_optin,
+                     b->warps_per_block, &g.cls.block, &best_blocks))
+      return LZ_ERR_INVALID_ARG;
+    const uint64_t wpb = g.cls.block / 32;
+    uint64_t grid = div_up(g.chunks, wpb);
+    if (grid > static_cast<uint64_t>(best_blocks) * ctx->sms) grid = best_blocks * ctx->sms;
+    uint64_t rb_max = 0;  // a parking slot holds any item's largest record
+    for (const lz_params &q : g.ps)
+      rb_max = std::max<uint64_t>(rb_max, record_bound(q.chunk_bytes / q.symbol_bytes,
+                                                       q.symbol_bytes, off_bytes(q.window),
+                                                       q.min_match) +
+                                              q.symbol_bytes);
+    glz::CompressArgs &A = g.cls.args;
+    A.n_items = static_cast<uint32_t>(g.descs.size());
+    A.total_chunks = g.chunks;
+    A.sm = sm;
+    A.park_slots = kParkSlots;
+    A.park_slot_bytes = round16(rb_max + 16);
+    A.spin_limit = glz::kSpinLimit;
+    g.cls.grid = static_cast<unsigned>(grid);
+    clear_at.push_back(clear);
+    clear += kScratchHead + 8ull * g.chunks;
+    clear = (clear + 255) & ~static_cast<size_t>(255);
+    park_at.push_back(park);
+    park += static_cast<size_t>(A.park_slot_bytes) * kParkSlots * wpb * grid;
+    park = (park + 255) & ~static_cast<size_t>(255);
+  }
+  lz_status s = batch_alloc(b, kBufScratch, clear + park, &b->scratch);
   if (s != LZ_OK) return s;
+  std::vector<glz::BufDesc> descs;
+  std::vector<uint64_t> bases;
+  for (const Group &g : groups)
+    for (const glz::BufDesc &d : g.descs) {
+      descs.push_back(d);
+      bases.push_back(d.gbase);
+    }
   const glz::BufDesc *d_items = nullptr, *d_empty = nullptr;
   const uint64_t *d_base = nullptr;
   if ((s = batch_upload(b, kBufItems, descs, &d_items)) != LZ_OK) return s;
   if ((s = batch_upload(b, kBufBases, bases, &d_base)) != LZ_OK) return s;
   if ((s = batch_upload(b, kBufEmpties, empties, &d_empty)) != LZ_OK) return s;
-  glz::CompressArgs &A = b->cargs;
-  A.items = d_items;
-  A.item_base = d_base;
-  A.n_items = static_cast<uint32_t>(descs.size());
-  A.total_chunks = total;
-  A.sm = sm;
-  A.ticket = static_cast<uint32_t *>(b->scratch);
-  A.status = reinterpret_cast<unsigned long long *>(static_cast<uint8_t *>(b->scratch) +
-                                                     kScratchHead);
-  A.err = ctx->d_err;
-  A.park = static_cast<uint8_t *>(b->scratch) + park_at;
-  A.park_slots = kParkSlots;
-  A.park_slot_bytes = slot_bytes;
-  A.spin_limit = glz::kSpinLimit;
-  A.first_ticket = 0;
+  cudaError_t e = cudaSuccess;
+  const int sides = static_cast<int>(std::min<size_t>(groups.empty() ? 0 : groups.size() - 1,
+                                                      kBatchSides));
+  if (sides && !b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  for (int i = 0; i < sides && e == cudaSuccess; ++i) {
+    if (!b->side[i]) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
+    if (e == cudaSuccess && !b->join[i])
+      e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
+  }
+  if (e != cudaSuccess) return cuda_status(e);
+  b->classes.clear();
+  uint8_t *base = static_cast<uint8_t *>(b->scratch);
+  for (size_t i = 0; i < groups.size(); ++i) {
+    glz::CompressArgs &A = groups[i].cls.args;
+    A.items = d_items;
+    A.item_base = d_base;
+    d_items += groups[i].descs.size();
+    d_base += groups[i].descs.size();
+    A.ticket = reinterpret_cast<uint32_t *>(base + clear_at[i]);
+    A.status = reinterpret_cast<unsigned long long *>(base + clear_at[i] + kScratchHead);
+    A.park = base + clear + park_at[i];
+    b->classes.push_back(groups[i].cls);
+  }
   b->d_empty = d_empty;
   b->n_empty = static_cast<uint32_t>(empties.size());
-  b->nj = nj;
-  b->block = block;
-  b->grid = static_cast<unsigned>(grid);
-  b->clear_bytes = status_end;
+  b->clear_bytes = clear;
   return LZ_OK;
+}
+
+// Class i > 0 goes to side stream (i - 1) % kBatchSides: each is ordered
+// after what the caller's stream holds now, and the caller's stream after it.
+lz_status batch_run_compress(lz_ctx *ctx, lz_batch *b, cudaStream_t st) {
+  if (b->clear_bytes && cudaMemsetAsync(b->scratch, 0, b->clear_bytes, st) != cudaSuccess)
+    return LZ_ERR_CUDA;
+  cudaError_t e = cudaSuccess;
+  if (b->n_empty) e = glz::launch_batch_empties(b->d_empty, b->n_empty, st);
+  const size_t n = b->classes.size();
+  const size_t sides = n > 1 ? std::min<size_t>(n - 1, kBatchSides) : 0;
+  if (sides && e == cudaSuccess) e = cudaEventRecord(b->fork, st);
+  for (size_t i = 0; i < sides && e == cudaSuccess; ++i)
+    e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
+  for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+    BatchClass &c = b->classes[i];
+    c.args.err = ctx->d_err;
+    e = glz::launch_batch_class(c.args, c.S, c.nj, c.mask, c.block, c.grid,
+                                i == 0 ? st : b->side[(i - 1) % kBatchSides]);
+  }
+  // joined also after a failed launch: the side streams must not run on
+  // unordered, nor a capture be left forked
+  for (size_t i = 0; i < sides; ++i) {
+    cudaError_t j = cudaEventRecord(b->join[i], b->side[i]);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(st, b->join[i], 0);
+    if (e == cudaSuccess) e = j;
+  }
+  return cuda_status(e);
 }
 
 uint64_t header_u(const uint8_t *h, int at, int n) {
@@ -1312,6 +1408,7 @@ lz_status lz_batch_create_ex(lz_ctx *ctx, const lz_batch_item *items, uint32_t n
   if (s != LZ_OK) {
     for (DevBuf &d : b->bufs)
       if (d.p) cudaFreeAsync(d.p, b->stream);
+    batch_streams_free(b);
     delete b;
     return s;
   }
@@ -1344,11 +1441,8 @@ lz_status lz_batch_run(lz_ctx *ctx, lz_batch *b, lz_stream_t stream) {
     b->dargs.err = ctx->d_err;
     return cuda_status(glz::launch_decompress_batch(b->dargs, b->dblock, st));
   }
-  b->cargs.err = ctx->d_err;
-  if (b->clear_bytes && cudaMemsetAsync(b->scratch, 0, b->clear_bytes, st) != cudaSuccess)
-    return LZ_ERR_CUDA;
-  return cuda_status(glz::launch_compress_batch(b->cargs, b->d_empty, b->n_empty, b->nj,
-                                                b->block, b->grid, st));
+  std::lock_guard<std::mutex> lock(b->run_mu);
+  return batch_run_compress(ctx, b, st);
 }
 
 void lz_batch_destroy(lz_batch *b, lz_stream_t stream) {
@@ -1357,6 +1451,7 @@ void lz_batch_destroy(lz_batch *b, lz_stream_t stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   for (DevBuf &d : b->bufs)
     if (d.p) cudaFreeAsync(d.p, st);
+  batch_streams_free(b);
   delete b;
 }
 
