@@ -1,0 +1,10 @@
+// compress_coop_s2.cu -- instances of the block-per-chunk compression
+// kernel for 2-byte symbols.
+#include "compress_coop_launch.cuh"
+
+namespace glz {
+cudaError_t launch_coop_s2(const CompressArgs &A, uint32_t nw, unsigned grid,
+                           cudaStream_t stream) {
+  return launch_coop_t<2>(A, nw, grid, stream);
+}
+}  // namespace glz

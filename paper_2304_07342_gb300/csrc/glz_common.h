@@ -64,6 +64,45 @@ struct CompressSmem {
   uint32_t hash_log2;  // hash table entries = 1 << hash_log2 (u16 each)
 };
 
+// Block of the compressor for few chunks (compress_coop.cuh): eight warps on
+// one chunk.  Byte offsets of its shared memory after the staged chunk.
+constexpr uint32_t kCoopWarps = 8;
+struct CoopSmem {
+  uint32_t planes_off;  // planes of the whole chunk, later the record's payload
+  uint32_t rows_off;    // rows of each warp
+  uint32_t info_off;    // per position: match length and offset (4 bytes)
+  uint32_t reach_off;   // per position: tokens visited in its slab (4 bytes)
+  uint32_t leave_off;   // per position: position after the slab (2 bytes)
+  uint32_t slab_off;    // three words per slab
+  uint32_t slabs;
+  uint32_t flags_off;
+  uint32_t total;
+};
+__host__ __device__ inline CoopSmem coop_layout(uint32_t S, uint32_t C, uint32_t nw) {
+  const uint32_t k = C / S;
+  CoopSmem L{};
+  L.slabs = (k + 31) / 32;
+  const uint32_t kk = 32 * L.slabs;  // whole slabs
+  uint32_t at = (C + 31) & ~15u;
+  L.planes_off = at;
+  at += L.slabs * mask_plane_words(S) * 4 + 16;  // (>= C + 16)
+  L.rows_off = at;
+  at += kCoopWarps * mask_rows_bytes(nw);
+  L.info_off = at;
+  at += 4 * kk;
+  L.reach_off = at;
+  at += 4 * kk;
+  L.leave_off = at;
+  at += 2 * kk;
+  L.slab_off = at;
+  at += 12 * L.slabs;
+  at = (at + 15) & ~15u;
+  L.flags_off = at;
+  at += 4 * L.slabs + 16;
+  L.total = (at + 127) & ~127u;
+  return L;
+}
+
 // One buffer to compress (one stream): per-buffer parameters and places.
 struct BufDesc {
   const uint8_t *in;
@@ -87,6 +126,7 @@ struct CompressArgs {
   uint32_t n_items;            // non-empty items
   uint64_t total_chunks;       // chunks over all items
   CompressSmem sm;             // per-warp layout (covers every item)
+  CoopSmem coop;               // or the layout of a block per chunk
   unsigned long long *status;  // one look-back word per chunk (cleared per call)
   uint32_t *ticket;            // work counter (cleared per call)
   uint32_t *err;               // sticky error bits

@@ -21,6 +21,9 @@ cudaError_t launch_compress_s2(const CompressArgs &A, uint32_t nj, int block,
 cudaError_t launch_compress_s4(const CompressArgs &A, uint32_t nj, int block,
                                unsigned grid, cudaStream_t stream);
 cudaError_t launch_decompress(DecompressArgs A, int block, cudaStream_t stream);
+cudaError_t launch_coop_s1(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
+cudaError_t launch_coop_s2(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
+cudaError_t launch_coop_s4(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
 cudaError_t launch_batch_empties(const BufDesc *empties, uint32_t n, cudaStream_t stream);
 cudaError_t launch_batch_class(const CompressArgs &A, uint32_t S, uint32_t nj, bool mask,
                                int block, unsigned grid, cudaStream_t stream);
@@ -218,6 +221,27 @@ bool block_shape(int64_t per_warp, int smem_per_sm, int smem_reserved, int smem_
     }
   }
   return best_warps > 0;
+}
+
+// Does a launch over `chunks` chunks take a block of eight warps per chunk
+// (compress_coop.cuh)?  When they would fill less than half of the warps that
+// one warp per chunk keeps resident, and the block fits: below that line a
+// launch lasts as long as one chunk.  Gives the layout for chunks of C bytes
+// and windows of 32 * nw symbols.
+bool coop_takes(const lz_ctx *ctx, uint64_t chunks, uint64_t resident_warps, uint32_t S,
+                uint32_t C, uint32_t nw, glz::CoopSmem *out) {
+  if (2 * chunks > resident_warps) return false;
+  *out = glz::coop_layout(S, C, nw);
+  return static_cast<int64_t>(out->total) + 1024 <= ctx->smem_optin && C / S <= 0x7E00;  // positions and the flag in 16 bits
+}
+
+cudaError_t launch_coop(const glz::CompressArgs &A, uint32_t S, uint32_t nw, unsigned grid,
+                        cudaStream_t st) {
+  switch (S) {
+    case 1: return glz::launch_coop_s1(A, nw, grid, st);
+    case 2: return glz::launch_coop_s2(A, nw, grid, st);
+    default: return glz::launch_coop_s4(A, nw, grid, st);
+  }
 }
 
 lz_status cuda_status(cudaError_t e) {
@@ -474,6 +498,12 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
   A.end_chunk = static_cast<uint32_t>(c1);
   uint32_t nj = 1;
   while (32 * nj < p->window) nj *= 2;
+  // (a caller's launch shape and the pieces of lz_compress_host keep one warp
+  // per chunk)
+  if (!warps_per_block && c0 == 0 && c1 == nc &&
+      glz::mask_parse_takes(S, p->window, p->min_match, A.buf.match) &&
+      coop_takes(ctx, nc, wpb * best_blocks * ctx->sms, S, C, std::max(nj, 4u), &A.coop))
+    return cuda_status(launch_coop(A, S, std::max(nj, 4u), static_cast<unsigned>(nc), st));
   const unsigned g = static_cast<unsigned>(grid);
   switch (S) {
     case 1: e = glz::launch_compress_s1(A, nj, block, g, st); break;
@@ -964,7 +994,7 @@ struct DevBuf {
 // one parse (masks or chains) and one range of windows.
 struct BatchClass {
   uint32_t S = 1, nj = 4;
-  bool mask = false;
+  bool mask = false, coop = false;
   int block = 32;
   unsigned grid = 1;
   glz::CompressArgs args{};
@@ -1175,6 +1205,13 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
     A.park_slot_bytes = round16(rb_max + 16);
     A.spin_limit = glz::kSpinLimit;
     g.cls.grid = static_cast<unsigned>(grid);
+    uint32_t c_max = 0;
+    for (const lz_params &q : g.ps) c_max = std::max(c_max, q.chunk_bytes);
+    if (g.cls.mask && !b->warps_per_block &&
+        coop_takes(ctx, g.chunks, wpb * best_blocks * ctx->sms, g.cls.S, c_max, g.cls.nj, &A.coop)) {
+      g.cls.coop = true;
+      g.cls.grid = static_cast<unsigned>(g.chunks);
+    }
     clear_at.push_back(clear);
     clear += kScratchHead + 8ull * g.chunks;
     clear = (clear + 255) & ~static_cast<size_t>(255);
@@ -1240,8 +1277,9 @@ lz_status batch_run_compress(lz_ctx *ctx, lz_batch *b, cudaStream_t st) {
   for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
     BatchClass &c = b->classes[i];
     c.args.err = ctx->d_err;
-    e = glz::launch_batch_class(c.args, c.S, c.nj, c.mask, c.block, c.grid,
-                                i == 0 ? st : b->side[(i - 1) % kBatchSides]);
+    const cudaStream_t on = i == 0 ? st : b->side[(i - 1) % kBatchSides];
+    e = c.coop ? launch_coop(c.args, c.S, c.nj, c.grid, on)
+               : glz::launch_batch_class(c.args, c.S, c.nj, c.mask, c.block, c.grid, on);
   }
   // joined also after a failed launch: the side streams must not run on
   // unordered, nor a capture be left forked

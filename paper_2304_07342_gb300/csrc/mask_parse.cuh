@@ -115,7 +115,8 @@ __device__ __forceinline__ uint32_t lowest_bit(const uint32_t (&v)[NW]) {
   return at + __ffs(w);
 }
 
-template <int S, int NW>
+// WHOLE: planes of every slab of the chunk are kept, else of the last 2 * NW.
+template <int S, int NW, bool WHOLE = false>
 struct MaskParser {
   using Sym = typename SymType<S>::T;
   static constexpr uint32_t kPlanes = mask_plane_words(S);  // plane words per slab
@@ -126,6 +127,12 @@ struct MaskParser {
   uint32_t k, act, ngroups, lane;
   uint32_t lift0[8];  // the first eight varying bits, see next_lifts
   uint32_t *planes, *rows;
+
+  // Plane words of slab n - t (any slab's when it lies before the chunk).
+  __device__ __forceinline__ uint32_t *slab_planes(uint32_t n, uint32_t t) const {
+    if constexpr (WHOLE) return planes + (t <= n ? n - t : 0u) * kPlanes;
+    else return planes + ((n - t) & (kRing - 1)) * kPlanes;
+  }
 
   __device__ __forceinline__ uint32_t symbol(uint32_t p) const {
     return p < k ? static_cast<uint32_t>(reinterpret_cast<const Sym *>(inb)[p]) : 0u;
@@ -187,15 +194,15 @@ struct MaskParser {
       own[b] = __ballot_sync(kFull, t < 0);
       my[b] = static_cast<uint32_t>(t >> 31);
     }
-    uint32_t *at = planes + 8 * group + FIRST;
-    if (lane == 0) store_row<N>(at + (n & (kRing - 1)) * kPlanes, own);
+    const uint32_t at = 8 * group + FIRST;
+    if (lane == 0) store_row<N>(slab_planes(n, 0) + at, own);
     if (!want_rows) return;
 #pragma unroll
     for (int b = 0; b < N; ++b) acc[0] &= ~(own[b] ^ my[b]);
 #pragma unroll
     for (int t = 1; t <= NW; ++t) {
       uint32_t x[N];
-      load_row<N>(at + ((n - t) & (kRing - 1)) * kPlanes, x);
+      load_row<N>(slab_planes(n, t) + at, x);
 #pragma unroll
       for (int b = 0; b < N; ++b) acc[t] &= ~(x[b] ^ my[b]);
     }
@@ -255,6 +262,87 @@ struct MaskParser {
     for (int j = 0; j < NW; ++j) a[j] &= e[j];
   }
 };
+
+// The longest match of the position p of this lane (place r of its slab) when
+// p >= from: its length (0: none of m symbols) and nearest offset; a = the
+// offsets that match over that length.  `open`: it still matches at the last
+// row kept and may be longer.
+template <int S, int NW, bool WHOLE>
+__device__ __forceinline__ void longest_match(const MaskParser<S, NW, WHOLE> &P, uint32_t p,
+                                              uint32_t r, uint32_t cur, uint32_t m, uint32_t M,
+                                              uint32_t W, bool overlap, uint32_t (&a)[NW],
+                                              uint32_t &len, uint32_t &off, bool &open) {
+  const uint32_t k = P.k;
+  len = 0;
+  off = 0;
+  open = false;
+  P.row(p, a);
+  if (W != 32u * NW) {
+#pragma unroll
+    for (int j = 0; j < NW; ++j)
+      a[j] &= W >= 32u * (j + 1) ? kFull : W <= 32u * j ? 0u : (1u << (W - 32u * j)) - 1u;
+  }
+  if (m >= 2) P.and_row(p + 1, a);
+  if (m >= 3) P.and_row(p + 2, a);
+#pragma unroll 1
+  for (uint32_t l = 3; l < m; ++l) P.and_row(p + l, a);
+  if (!overlap) a[0] &= kFull << (m - 1);
+  if (p >= cur && p + m <= k && any_bit<NW>(a)) {
+    const uint32_t lim = min(M, k - p), stop = min(lim, 64 - r), stop0 = min(stop, 32u);
+    uint32_t l = m;
+    bool more = true;
+#pragma unroll 1
+    while (l < stop0) {
+      uint32_t e[NW];
+      P.row(p + l, e);
+#pragma unroll
+      for (int j = 0; j < NW; ++j) e[j] &= a[j];
+      if (!overlap) e[0] &= kFull << l;
+      if (!any_bit<NW>(e)) {
+        more = false;
+        break;
+      }
+#pragma unroll
+      for (int j = 0; j < NW; ++j) a[j] = e[j];
+      ++l;
+    }
+#pragma unroll 1
+    while (more && l < stop) {
+      uint32_t e[NW];
+      P.row(p + l, e);
+      drop_offsets<NW>(e, overlap ? 0u : l);
+#pragma unroll
+      for (int j = 0; j < NW; ++j) e[j] &= a[j];
+      if (!any_bit<NW>(e)) {
+        more = false;
+        break;
+      }
+#pragma unroll
+      for (int j = 0; j < NW; ++j) a[j] = e[j];
+      ++l;
+    }
+    len = l;
+    off = lowest_bit<NW>(a);
+    open = more && l < lim;
+  }
+}
+
+// The greedy parse of a slab from each of its positions: `tok` = the lanes
+// of the token starts it visits, `last` = the lane of the last of them.  A
+// lane's successor is the lane of the next token start (itself when that lies
+// past the slab); joining the sets reached by the successors, twice as far
+// each time, takes five rounds of two shuffles (following one pointer after
+// the other took 20 instructions each).
+__device__ __forceinline__ void parse_from_every_lane(uint32_t step, uint32_t lane, uint32_t &tok,
+                                                      uint32_t &last) {
+  last = step <= lane ? lane - step : lane;
+  tok = 1u << lane;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    tok |= __shfl_sync(kFull, tok, last);
+    last = __shfl_sync(kFull, last, last);
+  }
+}
 
 // The greedy parse (section 2.2 steps 1-6) of the staged chunk of k symbols
 // and the record it gives: the flags are left in `flags`, the payload (and a
@@ -339,74 +427,15 @@ __device__ __forceinline__ void mask_parse(uint8_t *inb, uint32_t k, uint32_t ta
     if (cur >= 32 * (s + 1)) continue;  // the slab lies inside a pointer
     const uint32_t p = 32 * s + r;
 
-    // the longest match of every position from `cur` on: a = the offsets of
-    // matches of length >= len that may be that long
-    uint32_t a[NW];
-    P.row(p, a);
-    if (W != 32u * NW) {
-#pragma unroll
-      for (int j = 0; j < NW; ++j)
-        a[j] &= W >= 32u * (j + 1) ? kFull : W <= 32u * j ? 0u : (1u << (W - 32u * j)) - 1u;
-    }
-    if (m >= 2) P.and_row(p + 1, a);
-    if (m >= 3) P.and_row(p + 2, a);
-#pragma unroll 1
-    for (uint32_t l = 3; l < m; ++l) P.and_row(p + l, a);
-    if (!overlap) a[0] &= kFull << (m - 1);
-    uint32_t len = 0, off = 0;
-    bool open = false;  // still matching at the last row kept
-    if (p >= cur && p + m <= k && any_bit<NW>(a)) {
-      const uint32_t lim = min(M, k - p), stop = min(lim, 64 - r), stop0 = min(stop, 32u);
-      uint32_t l = m;
-      bool more = true;
-#pragma unroll 1
-      while (l < stop0) {
-        uint32_t e[NW];
-        P.row(p + l, e);
-#pragma unroll
-        for (int j = 0; j < NW; ++j) e[j] &= a[j];
-        if (!overlap) e[0] &= kFull << l;
-        if (!any_bit<NW>(e)) {
-          more = false;
-          break;
-        }
-#pragma unroll
-        for (int j = 0; j < NW; ++j) a[j] = e[j];
-        ++l;
-      }
-#pragma unroll 1
-      while (more && l < stop) {
-        uint32_t e[NW];
-        P.row(p + l, e);
-        drop_offsets<NW>(e, overlap ? 0u : l);
-#pragma unroll
-        for (int j = 0; j < NW; ++j) e[j] &= a[j];
-        if (!any_bit<NW>(e)) {
-          more = false;
-          break;
-        }
-#pragma unroll
-        for (int j = 0; j < NW; ++j) a[j] = e[j];
-        ++l;
-      }
-      len = l;
-      off = lowest_bit<NW>(a);
-      open = more && l < lim;
-    }
+    uint32_t a[NW], len, off;
+    bool open;
+    longest_match(P, p, r, cur, m, M, W, overlap, a, len, off, open);
 
-    // the parse through the slab from `cur`: a lane's successor is the lane
-    // of the next token start (itself when that lies past the slab); joining
-    // the sets reached by the successors, twice as far each time, gives every
-    // lane the lanes its parse would visit (five rounds of two shuffles; one
-    // pointer after the other took 20 instructions each)
+    // the parse through the slab from `cur`
     const uint32_t has = __ballot_sync(kFull, len != 0), opened = __ballot_sync(kFull, open);
     const uint32_t step = len ? len : 1u;
-    uint32_t next = step <= lane ? lane - step : lane, tok = 1u << lane;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-      tok |= __shfl_sync(kFull, tok, next);
-      next = __shfl_sync(kFull, next, next);
-    }
+    uint32_t tok, last;
+    parse_from_every_lane(step, lane, tok, last);
     tok = __shfl_sync(kFull, tok, 31 - (cur - 32 * s));
     const uint32_t ptr = tok & has;
     const uint32_t lv = __ffs(tok) - 1;  // lane of the last token

@@ -2,16 +2,19 @@
 matches that end around the rows it keeps (two slabs of 32 positions) or run
 on far past them, every number of varying symbol bits, windows that are not
 whole words, chunk lengths around a slab, the parameters at the edge of its
-route, and stored chunks whose input the record was written over.  Streams
-are compared byte for byte."""
+route, and stored chunks whose input the record was written over.  Every case
+runs with one warp per chunk (a stated launch shape) and with a block per
+chunk (what few chunks take).  Streams are compared byte for byte."""
 from __future__ import annotations
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2304_07342_gb300 import lz
 from tests import gpu_util as G
+from tests import test_gpu_literal_precheck as precheck
 
 pytestmark = pytest.mark.gpu
 
@@ -25,14 +28,25 @@ def codec():
     c.close()
 
 
-def _check(codec, x, S, C, W, m, M=255, version=1, overlap=False):
+def _compress(codec, d, P, wpb, match=lz.LZ_MATCH_EXACT, version=1):
+    out = torch.empty(lz.lz_compressed_bound(d.numel(), P), dtype=torch.uint8, device="cuda")
+    nb = torch.zeros(1, dtype=torch.int64, device="cuda")
+    lz.lz_compress_ex(codec.ctx, d.data_ptr(), d.numel(), P, out.data_ptr(), out.numel(),
+                      nb.data_ptr(), torch.cuda.current_stream().cuda_stream, match=match,
+                      version=version, warps_per_block=wpb)
+    assert codec.sync() == lz.LZ_OK
+    return out[:int(nb.item())].cpu().numpy()
+
+
+def _check(codec, x, S, C, W, m, M=255, version=1, overlap=False, offset=0):
     match = lz.LZ_MATCH_OVERLAP if overlap else lz.LZ_MATCH_EXACT
     mode = oracle.MATCH_OVERLAP if overlap else oracle.MATCH_EXACT
     ref = oracle.compress(x, oracle.Params(S, C, W, m, M), mode=mode, version=version)
-    d = G.to_dev(x)
-    got = codec.compress_sync(d, lz.Params(S, C, W, m, M), match=match, version=version).cpu().numpy()
-    assert np.array_equal(got, ref), G.first_difference(got, ref)
-    assert np.array_equal(G.gpu_decompress(codec, got), np.asarray(x).view(np.uint8).reshape(-1))
+    d = G.to_dev(x, offset)
+    for wpb in (0, 1):
+        got = _compress(codec, d, lz.Params(S, C, W, m, M), wpb, match, version)
+        assert np.array_equal(got, ref), (wpb, G.first_difference(got, ref))
+    assert np.array_equal(G.gpu_decompress(codec, ref), np.asarray(x).view(np.uint8).reshape(-1))
 
 
 def _random(n, S, seed, bits=None):
@@ -90,8 +104,61 @@ def test_stored_chunks_with_pointers(codec, S):
         x[at:at + 3] = x[at - 100:at - 97]
     raw = np.concatenate([x.view(np.uint8), np.arange(S - 1, dtype=np.uint8)])
     for offset in (0, 1):
-        d = G.to_dev(raw, offset)
-        P = lz.Params(S, 4096, 128, 3)
-        got = codec.compress_sync(d, P, version=2).cpu().numpy()
-        ref = oracle.compress(raw, oracle.Params(S, 4096, 128, 3, 255), version=2)
-        assert np.array_equal(got, ref), G.first_difference(got, ref)
+        _check(codec, raw, S, 4096, 128, 3, version=2, offset=offset)
+
+
+@pytest.mark.parametrize("case", precheck.CASES[::3])
+def test_literal_precheck_one_warp_per_chunk(codec, case):
+    """The pre-check's planted repeats with the launch that has one."""
+    S, C, W, m, target, d, length = case
+    x = precheck.distinct_random(2 * (C // S) + 11, S, seed=target + d)
+    at = C // S + target
+    n = max(0, min(length, 2 * (C // S) - at))
+    for i in range(n):
+        if target - d + i >= 0:
+            x[at + i] = x[at - d + i]
+    _check(codec, x, S, C, W, m)
+
+
+@pytest.mark.parametrize("S,C,W,m", [(1, 4096, 128, 3), (2, 4096, 128, 3), (4, 4096, 256, 2)])
+def test_either_side_of_the_line(codec, S, C, W, m):
+    """Sizes around the line between a block and a warp per chunk: the
+    streams of the two launches are the same bytes."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for chunks in (sms * 10, sms * 14, sms * 20):
+        r = np.random.default_rng(chunks)
+        v = r.integers(0, 40, chunks * C // S + 5)
+        x = np.repeat(v, r.integers(1, 4, v.size))[:v.size].astype(DT[S])
+        d = G.to_dev(x)
+        P = lz.Params(S, C, W, m)
+        a, b = _compress(codec, d, P, 0), _compress(codec, d, P, 1)
+        assert np.array_equal(a, b)
+
+
+def test_batch_with_many_chunks(codec):
+    """A batch whose classes fill the GPU with one warp per chunk, and one
+    small class beside them: every item equals its own call."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    params = [lz.Params(1, 2048, 64, 3), lz.Params(2, 2048, 128, 3), lz.Params(4, 2048, 256, 2),
+              lz.Params(1, 2048, 512, 3), lz.Params(2, 2048, 1024, 3), lz.Params(2, 2048, 128, 3)]
+    r = np.random.default_rng(0)
+    ins, outs, desc = [], [], []
+    nbs = torch.zeros(len(params), dtype=torch.int64, device="cuda")
+    for i, P in enumerate(params):
+        n = (sms * 20 if i != 3 else 40) * 2048 // P.S + 3
+        v = r.integers(0, 40, n)
+        x = np.repeat(v, r.integers(1, 4, n))[:n].astype(DT[P.S])
+        ins.append(G.to_dev(x))
+        outs.append(torch.zeros(lz.lz_compressed_bound(x.nbytes, P), dtype=torch.uint8, device="cuda"))
+        desc.append((ins[i].data_ptr(), x.nbytes, outs[i].data_ptr(), outs[i].numel(),
+                     nbs.data_ptr() + 8 * i, P))
+    st = torch.cuda.current_stream().cuda_stream
+    b = lz.lz_batch_create(codec.ctx, desc, stream=st)
+    try:
+        for _ in range(2):
+            lz.lz_batch_run(codec.ctx, b, st)
+        assert codec.sync() == lz.LZ_OK
+        for d, o, n, P in zip(ins, outs, nbs.tolist(), params):
+            assert np.array_equal(o[:n].cpu().numpy(), _compress(codec, d, P, 1))
+    finally:
+        lz.lz_batch_destroy(b, st)
