@@ -122,6 +122,7 @@ struct MaskParser {
   static constexpr uint32_t kPlanes = mask_plane_words(S);  // plane words per slab
   static constexpr uint32_t kRing = 2 * NW;                 // slabs of planes kept
   static constexpr uint32_t kRows = 64;                     // rows kept: two slabs
+  static constexpr uint32_t kPart = NW < 4 ? NW : 4;        // words of a row side by side
 
   const uint8_t *inb;
   uint32_t k, act, ngroups, lane;
@@ -246,14 +247,39 @@ struct MaskParser {
       uint32_t e[NW];
 #pragma unroll
       for (int j = 0; j < NW; ++j) e[j] = __funnelshift_rc(acc[j], acc[j + 1], lane + 1);
-      store_row<NW>(rows + (p & (kRows - 1)) * NW, e);
+      set_row(p, e);
     }
     __syncwarp();
   }
 
-  // E(p), a position of the last two slabs made with rows.
+  // E(p), a position of the last two slabs made with rows.  Rows of more than
+  // four words are split into parts of 16 bytes, part-major: neighbouring
+  // lanes then read neighbouring 16 bytes (whole rows of 32 and 64 bytes put
+  // the lanes of a 16-byte access 2 and 4 deep on the same banks).
   __device__ __forceinline__ void row(uint32_t p, uint32_t (&e)[NW]) const {
-    load_row<NW>(rows + (p & (kRows - 1)) * NW, e);
+    const uint32_t *at = rows + (p & (kRows - 1)) * kPart;
+    if constexpr (NW <= 4) {
+      load_row<NW>(at, e);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NW; j += 4) {
+        const uint4 t = *reinterpret_cast<const uint4 *>(at + j * kRows);
+        e[j] = t.x;
+        e[j + 1] = t.y;
+        e[j + 2] = t.z;
+        e[j + 3] = t.w;
+      }
+    }
+  }
+  __device__ __forceinline__ void set_row(uint32_t p, const uint32_t (&e)[NW]) const {
+    uint32_t *at = rows + (p & (kRows - 1)) * kPart;
+    if constexpr (NW <= 4) {
+      store_row<NW>(at, e);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NW; j += 4)
+        *reinterpret_cast<uint4 *>(at + j * kRows) = make_uint4(e[j], e[j + 1], e[j + 2], e[j + 3]);
+    }
   }
   __device__ __forceinline__ void and_row(uint32_t p, uint32_t (&a)[NW]) const {
     uint32_t e[NW];
