@@ -383,6 +383,7 @@ __device__ __forceinline__ bool decode_tokens(const Header &h, const uint8_t *pa
   // a literal of the round or lies before it (2 to 3 turns on codes with 50
   // to 80 % pointer symbols).
   uint32_t carry = 0;  // offset owning the previous round's last position
+  if (lane == 0) sl.dist[kRound] = 0;
 #pragma unroll 1
   for (uint32_t r0 = 0; r0 < k; r0 += kRound) {
     const uint32_t x0 = kPer * lane, j = r0 + x0;
@@ -427,19 +428,20 @@ __device__ __forceinline__ bool decode_tokens(const Header &h, const uint8_t *pa
     uint2 *mine = reinterpret_cast<uint2 *>(sl.dist + x0);
     *mine = make_uint2(__byte_perm(off[0], off[1], 0x5410), __byte_perm(off[2], off[3], 0x5410));
     __syncwarp();
-    // one turn: every source in the round moves to its own source
+    // one turn: every source in the round moves to its own source (by 0 at a
+    // literal; sources before the round read the 0 after the round's entries)
     auto turn = [&]() -> bool {
       uint32_t moved = 0;
 #pragma unroll
       for (uint32_t i = 0; i < kPer; ++i) {
-        uint32_t d = 0;
-        if (off[i] && f[i] >= r0) d = sl.dist[f[i] - r0];
+        const uint32_t d = sl.dist[min(f[i] - r0, kRound)];
         f[i] -= d;
         moved |= d;
       }
       return moved != 0;
     };
     bool again = true;
+#pragma unroll 1
     for (uint32_t n = 0; again && n < 4; ++n) again = turn();
     // long chains (matches that overlap their output): the distances already
     // followed replace the offsets, which doubles the reach of a turn.  A
@@ -453,20 +455,19 @@ __device__ __forceinline__ bool decode_tokens(const Header &h, const uint8_t *pa
       __syncwarp();
       again = turn();
     }
-    uint32_t any = 0;
-#pragma unroll
-    for (uint32_t i = 0; i < kPer; ++i) {
-      any |= off[i];
-      if (off[i] && GLZ_OK(f[i] < j + i)) v[i] = ld_slot<S>(ob, f[i], aligned);
-    }
-    // (a literal's slot is written again with its own value: other lanes of
-    // the round may be reading it)
+    // (a literal is read from and written to its own slot: other lanes of the
+    // round may be reading it)
     if constexpr (STAGED) {
-      if (any) st_slots<S>(ob, j, v);
+      if (nv) {
+#pragma unroll
+        for (uint32_t i = 0; i < kPer; ++i)
+          if (GLZ_OK(f[i] <= j + i)) v[i] = ld_slot<S>(ob, f[i], true);
+        st_slots<S>(ob, j, v);
+      }
     } else {
 #pragma unroll
       for (uint32_t i = 0; i < kPer; ++i)
-        if (off[i]) st_slot<S>(ob, j + i, v[i], aligned);
+        if (off[i] && GLZ_OK(f[i] < j + i)) st_slot<S>(ob, j + i, ld_slot<S>(ob, f[i], aligned), aligned);
     }
     __syncwarp();
   }

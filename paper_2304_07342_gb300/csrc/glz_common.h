@@ -193,7 +193,7 @@ struct DecodeLayout {
   uint32_t mark_bytes;
   uint32_t flags_off;  // flag bytes of one record (+ 16 slack)
   uint32_t flag_bytes;
-  uint32_t dist_off;   // 128 source distances (u16), one round of positions
+  uint32_t dist_off;   // 128 source distances (u16), one round of positions, and a zero
   uint32_t hi_off;     // k bytes (one-byte symbols, two-byte offsets) or none
   uint32_t io_off;     // output image + staged record
   uint32_t io_bytes;
@@ -228,7 +228,7 @@ __host__ __device__ inline DecodeLayout decode_layout(uint64_t kmax, uint64_t cm
   L.flag_bytes = static_cast<uint32_t>(((kmax + 7) / 8 + 15) & ~15ull) + 16;
   at += L.flag_bytes;
   L.dist_off = static_cast<uint32_t>(at);
-  at += 256;
+  at += 256 + 16;
   L.hi_off = static_cast<uint32_t>(at);
   if (hi) at += (kmax + 15) & ~15ull;
   const uint64_t base = at;
