@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
   const CoopSmem &L = A.coop;
   uint8_t *inb = smem, *pay = smem + L.planes_off;
   uint32_t *planes = reinterpret_cast<uint32_t *>(smem + L.planes_off);
-  uint32_t *rows = reinterpret_cast<uint32_t *>(smem + L.rows_off + warp * mask_rows_bytes(NW));
+  uint32_t *rows = reinterpret_cast<uint32_t *>(smem + L.rows_off + warp * mask_rows_bytes(NW, 1));
   uint32_t *info = reinterpret_cast<uint32_t *>(smem + L.info_off);    // length | offset << 8
   uint32_t *reach = reinterpret_cast<uint32_t *>(smem + L.reach_off);  // tokens of the slab
   uint16_t *leave = reinterpret_cast<uint16_t *>(smem + L.leave_off);  // position after it
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     P.planes = planes;
     P.rows = rows;
     P.find_varying_bits();
-    for (uint32_t n = warp; n < nslab; n += kCoopWarps) P.make_slab(n, false);
+    for (uint32_t n = warp; n < nslab; n += kCoopWarps) P.make_slabs(n, false);
     __syncthreads();
 
     // 2. longest matches and the parse through each slab
@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
 #pragma unroll 1
       for (uint32_t s = warp * per; s < s1; ++s) {
 #pragma unroll 1
-        while (made < nslab && made < s + 2) P.make_slab(made++, true);
+        while (made < nslab && made < s + 2) P.make_slabs(made++, true);
         const uint32_t p = 32 * s + r;
         uint32_t a[NW], len, off;
         bool open;

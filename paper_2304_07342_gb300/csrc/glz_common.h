@@ -40,14 +40,15 @@ __host__ __device__ inline bool mask_parse_takes(uint32_t S, uint32_t W, uint32_
          S * m >= 1u + (W <= 256 ? 1u : 2u);
 }
 // Plane words of one slab of 32 symbols (one per symbol bit) and, for windows
-// of 32 * nw symbols, the planes kept and the rows of two slabs and a spare
-// one (bytes).
+// of 32 * nw symbols, the planes kept and the rows of two slabs for each one
+// made at a time, and a spare row (bytes).
 __host__ __device__ constexpr uint32_t mask_plane_words(uint32_t S) { return 8 * S; }
 __host__ __device__ constexpr uint32_t mask_planes_bytes(uint32_t S, uint32_t nw) {
   return 2 * nw * mask_plane_words(S) * 4;
 }
-__host__ __device__ constexpr uint32_t mask_rows_bytes(uint32_t nw) {
-  return (65 * nw * 4 + 15) & ~15u;
+__host__ __device__ constexpr int mask_slabs_made(uint32_t nw) { return nw <= 8 ? 2 : 1; }
+__host__ __device__ constexpr uint32_t mask_rows_bytes(uint32_t nw, uint32_t made) {
+  return ((64 * made + 1) * nw * 4 + 15) & ~15u;
 }
 
 // Per-warp shared-memory layout of the compressor (byte offsets from the
@@ -87,7 +88,7 @@ __host__ __device__ inline CoopSmem coop_layout(uint32_t S, uint32_t C, uint32_t
   L.planes_off = at;
   at += L.slabs * mask_plane_words(S) * 4 + 16;  // (>= C + 16)
   L.rows_off = at;
-  at += kCoopWarps * mask_rows_bytes(nw);
+  at += kCoopWarps * mask_rows_bytes(nw, 1);
   L.info_off = at;
   at += 4 * kk;
   L.reach_off = at;

@@ -173,13 +173,14 @@ glz::CompressSmem compress_layout(const lz_params *p, uint32_t match) {
     // Bit planes in place of the links and rows in place of the payload area.
     // 1-byte symbols have no literal pre-check and take no more than these:
     // 14 KiB instead of 34 per warp at C = 8192, W = 512, 15 warps resident
-    // per SM instead of 6.  Others keep the chains' space (with one-byte
-    // links) for the pre-check's bitmap.
+    // per SM instead of 6.  Others keep at least the chains' space (with
+    // one-byte links) for the pre-check's bitmap.
     uint32_t nw = 4;  // (a batch runs small windows with 4 words)
     while (32 * nw < p->window) nw *= 2;
-    const uint32_t planes = glz::mask_planes_bytes(S, nw), rows = glz::mask_rows_bytes(nw);
-    links = S == 1 ? planes : std::max(planes, round16(k));
-    pay_region = S == 1 ? rows : std::max(rows, pay_region);
+    const uint32_t planes = glz::mask_planes_bytes(S, nw), rows = glz::mask_rows_bytes(nw, glz::mask_slabs_made(nw));
+    const uint32_t kept = S == 1 ? 0u : round16(k) + pay_region;
+    links = planes;
+    pay_region = std::max(rows, kept > planes ? kept - planes : 0u);
   }
   sm.prev_off = at;
   at += links;

@@ -116,12 +116,16 @@ __device__ __forceinline__ uint32_t lowest_bit(const uint32_t (&v)[NW]) {
 }
 
 // WHOLE: planes of every slab of the chunk are kept, else of the last 2 * NW.
+// COUNT: slabs made at a time; two share the plane words of the slabs before
+// them and the work around them (windows of 512 keep one: four slabs of their
+// rows would take the shared memory of three warps in thirteen).
 template <int S, int NW, bool WHOLE = false>
 struct MaskParser {
+  static constexpr int COUNT = WHOLE ? 1 : mask_slabs_made(NW);
   using Sym = typename SymType<S>::T;
   static constexpr uint32_t kPlanes = mask_plane_words(S);  // plane words per slab
-  static constexpr uint32_t kRing = 2 * NW;                 // slabs of planes kept
-  static constexpr uint32_t kRows = 64;                     // rows kept: two slabs
+  static constexpr uint32_t kRing = NW > 1 ? 2 * NW : 4;    // slabs of planes kept
+  static constexpr uint32_t kRows = 64 * COUNT;             // rows kept: two slabs, or four
   static constexpr uint32_t kPart = NW < 4 ? NW : 4;        // words of a row side by side
 
   const uint8_t *inb;
@@ -178,56 +182,73 @@ struct MaskParser {
     }
   }
 
-  // Planes FIRST .. FIRST + N - 1 of a group of eight of slab n: the plane
-  // words go to the ring, and acc[t] keeps the bits of slab n - t whose
-  // symbols agree with this lane's.  (A lane's bit as a mask comes from a
-  // multiplication and an arithmetic shift: selected by a predicate, the
-  // compiler turned each logic instruction below into two.)
+  // Planes FIRST .. FIRST + N - 1 of a group of eight of slabs n .. n + COUNT
+  // - 1: the plane words go to the ring, and acc[c][t] keeps the bits of slab
+  // n + c - t whose symbols agree with this lane's in slab n + c.  (A lane's
+  // bit as a mask comes from a multiplication and an arithmetic shift:
+  // selected by a predicate, the compiler turned each logic instruction below
+  // into two.)
   template <int FIRST, int N>
-  __device__ __forceinline__ void some_planes(uint32_t n, uint32_t group, uint32_t g,
+  __device__ __forceinline__ void some_planes(uint32_t n, uint32_t group,
+                                              const uint32_t (&g)[COUNT],
                                               const uint32_t (&lift)[8], bool want_rows,
-                                              uint32_t (&acc)[NW + 1]) const {
+                                              uint32_t (&acc)[COUNT][NW + 1]) const {
     static_assert(N == 2 || N == 4, "one vector store");
-    uint32_t my[N], own[N];
-#pragma unroll
-    for (int b = 0; b < N; ++b) {
-      const int32_t t = static_cast<int32_t>(g * lift[FIRST + b]);
-      own[b] = __ballot_sync(kFull, t < 0);
-      my[b] = static_cast<uint32_t>(t >> 31);
-    }
     const uint32_t at = 8 * group + FIRST;
-    if (lane == 0) store_row<N>(slab_planes(n, 0) + at, own);
+    uint32_t my[COUNT][N], own[COUNT][N];
+#pragma unroll
+    for (int c = 0; c < COUNT; ++c) {
+#pragma unroll
+      for (int b = 0; b < N; ++b) {
+        const int32_t t = static_cast<int32_t>(g[c] * lift[FIRST + b]);
+        own[c][b] = __ballot_sync(kFull, t < 0);
+        my[c][b] = static_cast<uint32_t>(t >> 31);
+      }
+      if (lane == 0) store_row<N>(slab_planes(n + c, 0) + at, own[c]);
+    }
     if (!want_rows) return;
 #pragma unroll
-    for (int b = 0; b < N; ++b) acc[0] &= ~(own[b] ^ my[b]);
+    for (int c = 0; c < COUNT; ++c)
+#pragma unroll
+      for (int o = 0; o <= c; ++o)
+#pragma unroll
+        for (int b = 0; b < N; ++b) acc[c][c - o] &= ~(own[o][b] ^ my[c][b]);
 #pragma unroll
     for (int t = 1; t <= NW; ++t) {
       uint32_t x[N];
       load_row<N>(slab_planes(n, t) + at, x);
 #pragma unroll
-      for (int b = 0; b < N; ++b) acc[t] &= ~(x[b] ^ my[b]);
+      for (int c = 0; c < COUNT; ++c)
+        if (t + c <= NW)
+#pragma unroll
+          for (int b = 0; b < N; ++b) acc[c][t + c] &= ~(x[b] ^ my[c][b]);
     }
   }
 
-  __device__ __forceinline__ void plane_group(uint32_t n, uint32_t group, uint32_t g,
+  __device__ __forceinline__ void plane_group(uint32_t n, uint32_t group,
+                                              const uint32_t (&g)[COUNT],
                                               const uint32_t (&lift)[8], bool want_rows,
-                                              uint32_t (&acc)[NW + 1]) const {
+                                              uint32_t (&acc)[COUNT][NW + 1]) const {
     some_planes<0, 4>(n, group, g, lift, want_rows, acc);
     // (codes around a mean vary in 5 to 7 Gray bits: the last pair is often idle)
     if (lift[4]) some_planes<4, 2>(n, group, g, lift, want_rows, acc);
     if (lift[6]) some_planes<6, 2>(n, group, g, lift, want_rows, acc);
   }
 
-  // Planes of slab n, and with `want_rows` the masks E(p) of its positions
-  // (for the full 32 * NW offsets; the window is applied by the reader).
-  __device__ __forceinline__ void make_slab(uint32_t n, bool want_rows) const {
+  // Planes of slabs n .. n + COUNT - 1, and with `want_rows` the masks E(p)
+  // of their positions (for the full 32 * NW offsets; the window is applied
+  // by the reader).
+  __device__ __forceinline__ void make_slabs(uint32_t n, bool want_rows) const {
     __syncwarp();  // rows and planes of the slabs these replace have been read
     const uint32_t p = 32 * n + 31 - lane;
-    const uint32_t v = symbol(p);
-    const uint32_t g = v ^ (v >> 1);
-    uint32_t acc[NW + 1];
+    uint32_t g[COUNT], acc[COUNT][NW + 1];
 #pragma unroll
-    for (int t = 0; t <= NW; ++t) acc[t] = kFull;
+    for (int c = 0; c < COUNT; ++c) {
+      const uint32_t v = symbol(p + 32 * c);
+      g[c] = v ^ (v >> 1);
+#pragma unroll
+      for (int t = 0; t <= NW; ++t) acc[c][t] = kFull;
+    }
     if (ngroups) plane_group(n, 0, g, lift0, want_rows, acc);
     if (ngroups > 1) {
       uint32_t rest = act, lift[8];
@@ -241,13 +262,18 @@ struct MaskParser {
     if (want_rows) {
       if (n < NW) {  // slabs before the chunk
 #pragma unroll
-        for (int t = 1; t <= NW; ++t)
-          if (static_cast<uint32_t>(t) > n) acc[t] = 0;
-      }
-      uint32_t e[NW];
+        for (int c = 0; c < COUNT; ++c)
 #pragma unroll
-      for (int j = 0; j < NW; ++j) e[j] = __funnelshift_rc(acc[j], acc[j + 1], lane + 1);
-      set_row(p, e);
+          for (int t = 1; t <= NW; ++t)
+            if (static_cast<uint32_t>(t) > n + c) acc[c][t] = 0;
+      }
+#pragma unroll
+      for (int c = 0; c < COUNT; ++c) {
+        uint32_t e[NW];
+#pragma unroll
+        for (int j = 0; j < NW; ++j) e[j] = __funnelshift_rc(acc[c][j], acc[c][j + 1], lane + 1);
+        set_row(p + 32 * c, e);
+      }
     }
     __syncwarp();
   }
@@ -381,7 +407,7 @@ __device__ __forceinline__ void parse_from_every_lane(uint32_t step, uint32_t la
 // made before the slab's tokens are written.  Requires m <= 32 and
 // W <= 32 * NW.
 //
-// The rows of two slabs are kept: a match that starts in slab s is followed
+// The rows of slabs s and s + 1 are kept: a match that starts in slab s is followed
 // through slab s + 1 by its own lane.  A longer one that the parse takes is
 // left open: its offsets wait in one more row, and the whole warp follows it
 // through the slabs after s + 1 as they are made.  It covers every position
@@ -416,8 +442,8 @@ __device__ __forceinline__ void mask_parse(uint8_t *inb, uint32_t k, uint32_t ta
   for (uint32_t s = 0; s < nslab; ++s) {
 #pragma unroll 1
     while (made < nslab && made < s + 2) {
-      P.make_slab(made, cur < 32 * (made + 1));
-      ++made;
+      P.make_slabs(made, cur < 32 * (made + P.COUNT));
+      made += P.COUNT;
     }
     if (long_p != kNone) {
       // the open match, through the rows of slabs s and s + 1
