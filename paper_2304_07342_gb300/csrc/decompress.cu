@@ -67,15 +67,20 @@ __device__ __forceinline__ bool read_header(const uint8_t *in, Header &h) {
   return ok;
 }
 
+// Eight bytes of the table or index: one load when the stream is 8-byte
+// aligned (`aligned`, the same for every thread), else byte by byte.
+__device__ __forceinline__ uint64_t ld_entry(const uint8_t *p, bool aligned) {
+  return aligned ? *reinterpret_cast<const uint64_t *>(p) : ld_le(p, 8);
+}
+
 // Sum of the record sizes of chunks [lo, hi) (hi - lo <= 64).
 __device__ __forceinline__ uint64_t record_bytes(const uint8_t *table,
                                                  uint32_t lo, uint32_t hi,
-                                                 uint32_t lane) {
+                                                 uint32_t lane, bool aligned) {
   uint64_t part = 0;
   for (uint32_t e = lo + lane; e < hi; e += 32) {
-    const uint64_t ntok = ld_le(table + 8ull * e, 4);
-    const uint64_t pay = ld_le(table + 8ull * e + 4, 4);
-    part += (ntok + 7) / 8 + pay;
+    const uint64_t v = ld_entry(table + 8ull * e, aligned);
+    part += ((v & 0xFFFFFFFFu) + 7) / 8 + (v >> 32);
   }
   return warp_sum_u64(part);
 }
@@ -501,17 +506,19 @@ __device__ __forceinline__ bool decode_chunk(const DecompressArgs &A, const Head
   const uint8_t *table = in + kHeaderBytes;
   const uint8_t *index = table + 8ull * h.nc;
   const uint32_t j = c / kIndexStride;
-  const uint64_t idxv = ld_le(index + 8ull * j, 8);
-  const uint64_t part = record_bytes(table, j * kIndexStride, c, lane);
+  const bool al = (reinterpret_cast<uintptr_t>(in) & 7u) == 0;
+  const uint64_t idxv = ld_entry(index + 8ull * j, al);
+  const uint64_t entry = ld_entry(table + 8ull * c, al);
+  const uint64_t part = record_bytes(table, j * kIndexStride, c, lane, al);
   bool bad = false;
   if (c == 0) bad = idxv != 0;
   if (c % kIndexStride == 0 && c > 0) {
-    const uint64_t prev = ld_le(index + 8ull * (j - 1), 8);
-    const uint64_t sb = record_bytes(table, c - kIndexStride, c, lane);
+    const uint64_t prev = ld_entry(index + 8ull * (j - 1), al);
+    const uint64_t sb = record_bytes(table, c - kIndexStride, c, lane, al);
     bad = bad || prev + sb != idxv;
   }
-  const uint32_t ntok = static_cast<uint32_t>(ld_le(table + 8ull * c, 4));
-  const uint32_t pay = static_cast<uint32_t>(ld_le(table + 8ull * c + 4, 4));
+  const uint32_t ntok = static_cast<uint32_t>(entry);
+  const uint32_t pay = static_cast<uint32_t>(entry >> 32);
   const uint64_t fb = (static_cast<uint64_t>(ntok) + 7) / 8;
   const uint64_t rec_at = records_at + idxv + part;
   const uint64_t chunk_at = static_cast<uint64_t>(c) * h.C;
@@ -549,9 +556,27 @@ __device__ __forceinline__ bool decode_chunk(const DecompressArgs &A, const Head
     }
     return true;
   }
-  // a chunk without pointers is its payload: copy it straight out
+  // the flag words are copied out (the output image grows from the start of
+  // the io area towards the record's flags), the bits past the last token
+  // cleared up to a round of the token phase
+  const uint32_t fwords = ((static_cast<uint32_t>(fb) + 15u) & ~15u) / 4;
+  if (!GLZ_OK(4 * fwords <= sl.flag_bytes)) return true;
   uint32_t any = 0;
-  for (uint32_t i = lane; i < fb; i += 32) any |= flags[i];
+  for (uint32_t i = lane; i < fwords; i += 32) {
+    uint32_t v = 0;
+    if (32 * i < ntok) {
+      if (sl.io) {
+        v = ld_u32_any(flags + 4 * i);
+      } else {
+        for (uint32_t q = 0; q < 4; ++q)
+          if (4 * i + q < fb) v |= static_cast<uint32_t>(flags[4 * i + q]) << (8 * q);
+      }
+      if (ntok - 32 * i < 32) v &= (1u << (ntok - 32 * i)) - 1u;
+    }
+    reinterpret_cast<uint32_t *>(sl.fl)[i] = v;
+    any |= v;
+  }
+  // a chunk without pointers is its payload: copy it straight out
   if (!__any_sync(kFull, any != 0)) {
     if (ntok != k || pay != bytes_c) {
       if (lane == 0) atomicOr(A.err, kErrCorrupt);
@@ -568,16 +593,6 @@ __device__ __forceinline__ bool decode_chunk(const DecompressArgs &A, const Head
   // the tail bytes, read before the output image may grow over the record
   const uint8_t tb = lane < tail ? payload[pay_tok + lane] : 0;
   bool ok;
-  // the flag bytes are copied out first (the output image grows from the
-  // start of the io area towards the record's flags), the bits past the last
-  // token cleared up to a round of the token phase
-  const uint32_t fpad = (static_cast<uint32_t>(fb) + 15u) & ~15u;
-  if (!GLZ_OK(fpad <= sl.flag_bytes)) return true;
-  for (uint32_t i = lane; i < fpad; i += 32) {
-    uint32_t v = i < fb ? flags[i] : 0u;
-    if (i + 1 == fb && (ntok & 7u)) v &= (1u << (ntok & 7u)) - 1u;
-    sl.fl[i] = static_cast<uint8_t>(v);
-  }
   __syncwarp();
   if (sl.io) {
     ok = decode_tokens_s<true>(h, payload, ntok, pay_tok, k, sl.io, true, sl, lane);
@@ -644,8 +659,12 @@ __global__ void __launch_bounds__(1024, 1) decompress_kernel(const DecompressArg
     fence_mbar_init();
   }
   __syncwarp();
-  const uint32_t gw = blockIdx.x * active + warp;
+  // chunks that do not fill the GPU spread over all SMs (block by block, 256
+  // chunks ran on 8: 1 MiB took 34.8 us, 19.0 spread); more go block by block
+  // (neighbouring chunks on one SM: 512 MiB of literal chunks 186 us, 190
+  // spread)
   const uint32_t nwarps = gridDim.x * active;
+  const uint32_t gw = h.nc < nwarps ? warp * gridDim.x + blockIdx.x : blockIdx.x * active + warp;
   for (uint32_t c = gw; c < h.nc; c += nwarps)
     if (!decode_chunk(A, h, c, records_at, sl, lane)) break;
   if (lane == 0) checked_fold(A.err);
@@ -676,7 +695,10 @@ __global__ void __launch_bounds__(1024, 1) decompress_batch_kernel(const Decompr
   }
   __syncwarp();
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * active;
-  for (uint64_t g = static_cast<uint64_t>(blockIdx.x) * active + warp; g < B.total_chunks;
+  // (few chunks spread over the SMs, as above)
+  for (uint64_t g = B.total_chunks < stride ? static_cast<uint64_t>(warp) * gridDim.x + blockIdx.x
+                                            : static_cast<uint64_t>(blockIdx.x) * active + warp;
+       g < B.total_chunks;
        g += stride) {
     uint32_t lo = 0, hi = B.n_items;
     while (hi - lo > 1) {
