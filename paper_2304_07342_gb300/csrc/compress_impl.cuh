@@ -7,8 +7,10 @@
 //   1. stages the chunk into its shared-memory slice (1-D TMA bulk copy);
 //   2. checks whether any position can start a match at all (a Bloom
 //      filter over symbol keys, tried after a chunk without pointers;
-//      chunks without repeats end here as all literals), else links every
-//      position to the last earlier position with the same hash of its
+//      chunks without repeats end here as all literals).  Exact matchers with
+//      windows up to 512 then take the parse by equality masks
+//      (mask_parse.cuh), which does step 3 and the record as well; the
+//      others link every position to the last earlier position with the same hash of its
 //      first min(m, 8/S) symbols (hash chains; __match_any_sync links
 //      positions of one 32-position slab) and marks the positions whose
 //      chain holds their key inside the window -- only those can start a
@@ -1169,17 +1171,20 @@ __device__ __forceinline__ uint32_t take_ticket(const CompressArgs &A, uint32_t 
   return __shfl_sync(kFull, t, 0);
 }
 
-// Register limit of a kernel, as resident blocks of 256 threads: the mask
-// parse left alone takes 140 registers, far past what the shared memory
-// would keep resident (28 warps per SM at C = 4096, S = 2; 23 at C = 4096,
-// S = 4, W = 256; 15 at C = 8192, W = 512).
-constexpr int min_blocks(int nj, bool mask) {
-  return mask ? (nj <= 4 ? 4 : nj <= 8 ? 3 : 2) : (nj < 32 ? 4 : 3);
+// Registers per thread.  The mask parse left alone takes 140, far more than
+// the shared memory would keep resident; the limits are what the register
+// file gives the warps that fit: 72 at windows up to 128 (28 warps per SM at
+// S = 2, C = 4096: 2,140 us for 256 MiB of quantization codes, 2,230 at 64
+// with spills, 2,185 at 80), 96 up to 256 (21 warps at S = 4, C = 4096: 860 us
+// for 128 MiB of Markov words, 925 at 80, 936 at 104), 128 up to 512 (15 warps
+// at S = 1, C = 8192).
+constexpr int reg_limit(int nj, bool mask) {
+  return mask ? (nj <= 4 ? 72 : nj <= 8 ? 96 : 128) : (nj < 32 ? 64 : 80);
 }
 
 // Single buffer: the symbol size is a template parameter.
 template <int S, int NJ, bool MASK>
-__global__ void __launch_bounds__(256, min_blocks(NJ, MASK)) compress_kernel(const CompressArgs A) {
+__global__ void __maxnreg__(reg_limit(NJ, MASK)) compress_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t lane = threadIdx.x & 31;
   WarpState W;
@@ -1215,8 +1220,7 @@ __device__ __forceinline__ uint32_t find_item(const CompressArgs &A, uint64_t g,
 // size, parse and range of windows) in order; each buffer carries its own
 // parameters, kept in shared memory while one of its chunks is compressed.
 template <int S, int NJ, bool MASK>
-__global__ void __launch_bounds__(256, min_blocks(NJ, MASK))
-    compress_batch_kernel(const CompressArgs A) {
+__global__ void __maxnreg__(reg_limit(NJ, MASK)) compress_batch_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ BufDesc descs[8];
   const uint32_t lane = threadIdx.x & 31;

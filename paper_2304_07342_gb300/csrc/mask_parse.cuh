@@ -188,10 +188,10 @@ struct MaskParser {
   // bit as a mask comes from a multiplication and an arithmetic shift:
   // selected by a predicate, the compiler turned each logic instruction below
   // into two.)
-  template <int FIRST, int N>
+  template <int FIRST, int N, bool ROWS>
   __device__ __forceinline__ void some_planes(uint32_t n, uint32_t group,
                                               const uint32_t (&g)[COUNT],
-                                              const uint32_t (&lift)[8], bool want_rows,
+                                              const uint32_t (&lift)[8],
                                               uint32_t (&acc)[COUNT][NW + 1]) const {
     static_assert(N == 2 || N == 4, "one vector store");
     const uint32_t at = 8 * group + FIRST;
@@ -206,7 +206,7 @@ struct MaskParser {
       }
       if (lane == 0) store_row<N>(slab_planes(n + c, 0) + at, own[c]);
     }
-    if (!want_rows) return;
+    if constexpr (!ROWS) return;
 #pragma unroll
     for (int c = 0; c < COUNT; ++c)
 #pragma unroll
@@ -225,20 +225,22 @@ struct MaskParser {
     }
   }
 
+  template <bool ROWS>
   __device__ __forceinline__ void plane_group(uint32_t n, uint32_t group,
                                               const uint32_t (&g)[COUNT],
-                                              const uint32_t (&lift)[8], bool want_rows,
+                                              const uint32_t (&lift)[8],
                                               uint32_t (&acc)[COUNT][NW + 1]) const {
-    some_planes<0, 4>(n, group, g, lift, want_rows, acc);
+    some_planes<0, 4, ROWS>(n, group, g, lift, acc);
     // (codes around a mean vary in 5 to 7 Gray bits: the last pair is often idle)
-    if (lift[4]) some_planes<4, 2>(n, group, g, lift, want_rows, acc);
-    if (lift[6]) some_planes<6, 2>(n, group, g, lift, want_rows, acc);
+    if (lift[4]) some_planes<4, 2, ROWS>(n, group, g, lift, acc);
+    if (lift[6]) some_planes<6, 2, ROWS>(n, group, g, lift, acc);
   }
 
-  // Planes of slabs n .. n + COUNT - 1, and with `want_rows` the masks E(p)
-  // of their positions (for the full 32 * NW offsets; the window is applied
-  // by the reader).
-  __device__ __forceinline__ void make_slabs(uint32_t n, bool want_rows) const {
+  // Planes of slabs n .. n + COUNT - 1, and with ROWS the masks E(p) of their
+  // positions (for the full 32 * NW offsets; the window is applied by the
+  // reader).
+  template <bool ROWS>
+  __device__ __forceinline__ void make_slabs(uint32_t n) const {
     __syncwarp();  // rows and planes of the slabs these replace have been read
     const uint32_t p = 32 * n + 31 - lane;
     uint32_t g[COUNT], acc[COUNT][NW + 1];
@@ -249,17 +251,17 @@ struct MaskParser {
 #pragma unroll
       for (int t = 0; t <= NW; ++t) acc[c][t] = kFull;
     }
-    if (ngroups) plane_group(n, 0, g, lift0, want_rows, acc);
+    if (ngroups) plane_group<ROWS>(n, 0, g, lift0, acc);
     if (ngroups > 1) {
       uint32_t rest = act, lift[8];
       next_lifts(rest, lift);
 #pragma unroll 1
       for (uint32_t group = 1; group < ngroups; ++group) {
         next_lifts(rest, lift);
-        plane_group(n, group, g, lift, want_rows, acc);
+        plane_group<ROWS>(n, group, g, lift, acc);
       }
     }
-    if (want_rows) {
+    if constexpr (ROWS) {
       if (n < NW) {  // slabs before the chunk
 #pragma unroll
         for (int c = 0; c < COUNT; ++c)
@@ -442,7 +444,7 @@ __device__ __forceinline__ void mask_parse(uint8_t *inb, uint32_t k, uint32_t ta
   for (uint32_t s = 0; s < nslab; ++s) {
 #pragma unroll 1
     while (made < nslab && made < s + 2) {
-      P.make_slabs(made, cur < 32 * (made + P.COUNT));
+      P.template make_slabs<true>(made);  // (also inside a long match: rare)
       made += P.COUNT;
     }
     if (long_p != kNone) {
