@@ -23,6 +23,65 @@
 
 namespace glz {
 
+// The literal pre-check of compress_impl.cuh (literal_chunk) by the whole
+// block: true only when no position of the chunk can start a match of >= m
+// symbols.  All keys are ORed into one Bloom filter of a word per position, in
+// no order between warps, so of two positions with one key the one ORed later
+// is flagged: a flagged position is checked exactly as the target of a match
+// and as the source of one, over the whole window.  Every thread returns the
+// same answer.  For each flagged position one more full scan than
+// literal_chunk's, but about one chunk in two has none.
+constexpr uint32_t kCoopMaxFlagged = 16;
+
+template <int S>
+__device__ __forceinline__ bool literal_chunk_block(const typename SymType<S>::T *sym, uint32_t k,
+                                                    const BufDesc &B, uint32_t *bm,
+                                                    uint32_t nwords, uint32_t *flagged,
+                                                    uint32_t *count, uint32_t warp,
+                                                    uint32_t lane) {
+  for (uint32_t i = threadIdx.x; i < nwords / 4; i += blockDim.x)
+    reinterpret_cast<uint4 *>(bm)[i] = make_uint4(0, 0, 0, 0);
+  if (threadIdx.x == 0) *count = 0;
+  __syncthreads();
+  const uint8_t *in = reinterpret_cast<const uint8_t *>(sym);
+  const uint32_t kb = S * min(B.m, 8u / S);  // key bytes, as in build_chains
+  const uint32_t mlo = kb >= 4 ? kFull : (1u << (8 * kb)) - 1u;
+  const uint32_t mhi = kb <= 4 ? 0u : (kb >= 8 ? kFull : (1u << (8 * (kb - 4))) - 1u);
+  const volatile uint32_t *seen = count;
+  for (uint32_t p0 = 32 * warp; p0 < k && *seen <= kCoopMaxFlagged; p0 += 32 * kCoopWarps) {
+    const uint32_t p = p0 + lane;
+    if (p + B.m > k) continue;
+    uint32_t lo, hi;
+    key_at<S>(in, p, mlo, mhi, lo, hi);
+    const uint32_t h = ((hi * 0x85EBCA77u) ^ lo) * 0x9E3779B1u, g = h * 0xC2B2AE3Du;
+    const uint32_t mask = (1u << (g >> 27)) | (1u << ((g >> 22) & 31u)) |
+                          (1u << ((g >> 17) & 31u)) | (1u << ((g >> 12) & 31u));
+    const uint32_t at = __umulhi(h, nwords);
+    if (GLZ_OK(at < nwords) && (atomicOr(&bm[at], mask) & mask) == mask) {
+      const uint32_t i = atomicAdd(count, 1u);
+      if (i < kCoopMaxFlagged) flagged[i] = p;
+    }
+  }
+  __syncthreads();
+  const uint32_t n = *count;
+  bool hit = n > kCoopMaxFlagged;
+  if (!hit) {
+    for (uint32_t i = warp; i < n && !hit; i += kCoopWarps) {
+      const uint32_t p = flagged[i];
+      hit = match_near<S>(sym, k, B, p, p + 1, lane);  // p as the target
+      bool eq_any = false;                             // p as the source
+      const uint32_t end = min(k, p + B.W + 1);
+      for (uint32_t q = p + 1 + lane; q < end; q += 32) {
+        bool eq = (q - p >= B.m || B.match == kMatchOverlap) && q + B.m <= k;
+        for (uint32_t x = 0; eq && x < B.m; ++x) eq = sym[q + x] == sym[p + x];
+        eq_any |= eq;
+      }
+      hit |= __any_sync(kFull, eq_any) != 0;
+    }
+  }
+  return !__syncthreads_or(hit);
+}
+
 template <int S, int NW>
 __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     compress_coop_kernel(const CompressArgs A) {
@@ -30,7 +89,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ BufDesc B;
   __shared__ __align__(8) uint64_t bar;
-  __shared__ uint32_t s_ticket, s_totals;
+  __shared__ uint32_t s_ticket, s_totals, s_flagged[kCoopMaxFlagged], s_count;
   __shared__ uint8_t *s_out;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const CoopSmem &L = A.coop;
@@ -50,6 +109,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     if (!A.items) B = A.buf;
   }
   uint32_t phase = 0;
+  bool try_literal = true;  // the block's previous chunk was all literals
   const uint64_t end_ticket = A.items ? A.total_chunks : A.end_chunk;
   while (true) {
     __syncthreads();
@@ -93,91 +153,99 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     staged = __syncthreads_and(staged);
     if (!staged && threadIdx.x == 0) atomicOr(A.err, kErrTimeout);
 
-    // 1. planes
-    MaskParser<S, NW, true> P;
-    P.inb = inb;
-    P.k = k;
-    P.lane = lane;
-    P.planes = planes;
-    P.rows = rows;
-    P.find_varying_bits();
-    for (uint32_t n = warp; n < nslab; n += kCoopWarps) P.make_slabs(n, false);
-    __syncthreads();
-
-    // 2. longest matches and the parse through each slab
+    // (tried after a chunk without pointers, as with one warp per chunk; the
+    // filter takes the place of `info`)
+    const bool literal = try_literal && literal_chunk_block<S>(
+        reinterpret_cast<const Sym *>(inb), k, B, info, 32 * nslab, s_flagged, &s_count, warp, lane);
     const bool overlap = B.match == kMatchOverlap;
     const uint32_t m = B.m, M = B.M, W = B.W, tsz = 1 + B.offB;
     const uint32_t r = 31 - lane;
-    {
-      const uint32_t per = (nslab + kCoopWarps - 1) / kCoopWarps;
-      const uint32_t s1 = min(nslab, (warp + 1) * per);
-      uint32_t made = warp * per;
-#pragma unroll 1
-      for (uint32_t s = warp * per; s < s1; ++s) {
-#pragma unroll 1
-        while (made < nslab && made < s + 2) P.make_slabs(made++, true);
-        const uint32_t p = 32 * s + r;
-        uint32_t a[NW], len, off;
-        bool open;
-        longest_match(P, p, r, 0, m, M, W, overlap, a, len, off, open);
-        const uint32_t step = len ? len : 1u;
-        uint32_t tok, last;
-        parse_from_every_lane(step, lane, tok, last);
-        const uint32_t out = 32 * s + 31 - last + __shfl_sync(kFull, step, last);
-        const uint32_t any = __ballot_sync(kFull, len != 0);
-        const uint32_t opened = __ballot_sync(kFull, open);
-        if (p < k) {
-          info[p] = len | (off << 8);
-          reach[p] = tok;
-          leave[p] = static_cast<uint16_t>(out | ((opened >> last) & 1u ? kOpen : 0u));
-        }
-        if (lane == 0) has[s] = any;
-      }
-    }
-    __syncthreads();
+    if (!literal) {
+      // 1. planes
+      MaskParser<S, NW, true> P;
+      P.inb = inb;
+      P.k = k;
+      P.lane = lane;
+      P.planes = planes;
+      P.rows = rows;
+      P.find_varying_bits();
+      for (uint32_t n = warp; n < nslab; n += kCoopWarps) P.template make_slabs<false>(n);
+      __syncthreads();
 
-    // 3. the parse from slab to slab; token and pointer counts before each
-    if (warp == 0) {
-      uint32_t cur = 0;
-      while (cur < k) {
-        const uint32_t s = cur >> 5, tok = reach[cur];
-        uint32_t next = leave[cur];
-        if (lane == 0) toks[s] = tok;
-        if (next & kOpen) {
-          const uint32_t q = 32 * s + 31 - (__ffs(tok) - 1);
-          uint32_t l, d;
-          window_match<S, NW>(reinterpret_cast<const Sym *>(inb), k, B, q, lane, l, d);
-          if (lane == 0) info[q] = l | (d << 8);
-          next = q + l;
+      // 2. longest matches and the parse through each slab
+      {
+        const uint32_t per = (nslab + kCoopWarps - 1) / kCoopWarps;
+        const uint32_t s1 = min(nslab, (warp + 1) * per);
+        uint32_t made = warp * per;
+#pragma unroll 1
+        for (uint32_t s = warp * per; s < s1; ++s) {
+#pragma unroll 1
+          while (made < nslab && made < s + 2) P.template make_slabs<true>(made++);
+          const uint32_t p = 32 * s + r;
+          uint32_t a[NW], len, off;
+          bool open;
+          longest_match(P, p, r, 0, m, M, W, overlap, a, len, off, open);
+          const uint32_t step = len ? len : 1u;
+          uint32_t tok, last;
+          parse_from_every_lane(step, lane, tok, last);
+          const uint32_t out = 32 * s + 31 - last + __shfl_sync(kFull, step, last);
+          const uint32_t any = __ballot_sync(kFull, len != 0);
+          const uint32_t opened = __ballot_sync(kFull, open);
+          if (p < k) {
+            info[p] = len | (off << 8);
+            reach[p] = tok;
+            leave[p] = static_cast<uint16_t>(out | ((opened >> last) & 1u ? kOpen : 0u));
+          }
+          if (lane == 0) has[s] = any;
         }
-        cur = next;
       }
-      __syncwarp();
-      uint32_t before = 0;  // tokens | pointers << 16
-      for (uint32_t b0 = 0; b0 < nslab; b0 += 32) {
-        const uint32_t s = b0 + lane;
-        uint32_t t = 0, x = 0;
-        if (s < nslab) {
-          t = toks[s];
-          if (k - 32 * s < 32) t &= kFull << (32 - (k - 32 * s));
-          toks[s] = t;
-          x = __popc(t) | (__popc(t & has[s]) << 16);
+      __syncthreads();
+
+      // 3. the parse from slab to slab; token and pointer counts before each
+      if (warp == 0) {
+        uint32_t cur = 0;
+        while (cur < k) {
+          const uint32_t s = cur >> 5, tok = reach[cur];
+          uint32_t next = leave[cur];
+          if (lane == 0) toks[s] = tok;
+          if (next & kOpen) {
+            const uint32_t q = 32 * s + 31 - (__ffs(tok) - 1);
+            uint32_t l, d;
+            window_match<S, NW>(reinterpret_cast<const Sym *>(inb), k, B, q, lane, l, d);
+            if (lane == 0) info[q] = l | (d << 8);
+            next = q + l;
+          }
+          cur = next;
         }
-        uint32_t total;
-        const uint32_t excl = warp_excl_scan(x, lane, total);
-        if (s < nslab) base[s] = before + excl;
-        before += total;
+        __syncwarp();
+        uint32_t before = 0;  // tokens | pointers << 16
+        for (uint32_t b0 = 0; b0 < nslab; b0 += 32) {
+          const uint32_t s = b0 + lane;
+          uint32_t t = 0, x = 0;
+          if (s < nslab) {
+            t = toks[s];
+            if (k - 32 * s < 32) t &= kFull << (32 - (k - 32 * s));
+            toks[s] = t;
+            x = __popc(t) | (__popc(t & has[s]) << 16);
+          }
+          uint32_t total;
+          const uint32_t excl = warp_excl_scan(x, lane, total);
+          if (s < nslab) base[s] = before + excl;
+          before += total;
+        }
+        if (lane == 0) s_totals = before;
       }
-      if (lane == 0) s_totals = before;
+      __syncthreads();
+
     }
-    __syncthreads();
 
     // 4. the record
-    uint32_t ntok = s_totals & 0xFFFFu;
-    const uint32_t np = s_totals >> 16;
+    uint32_t ntok = literal ? k : s_totals & 0xFFFFu;
+    const uint32_t np = literal ? 0u : s_totals >> 16;
+    try_literal = np == 0;
     uint32_t pb = S * (ntok - np) + tsz * np + tail, fb = (ntok + 7) / 8;
     const bool stored = B.version == 2 && fb + pb >= bytes;  // the chunk as it is
-    if (!stored) {
+    if (!stored && !literal) {
       const uint32_t earlier = lane == 31 ? 0u : kFull << (lane + 1);
       for (uint32_t s = warp; s < nslab; s += kCoopWarps) {
         const uint32_t tok = toks[s], ptr = tok & has[s], b = base[s];
@@ -186,7 +254,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
         const uint32_t t = (b & 0xFFFFu) + __popc(tok & earlier);
         const uint32_t q = (b >> 16) + __popc(ptr & earlier);
         const uint32_t p = 32 * s + r, po = S * (t - q) + tsz * q;
-        uint32_t v = P.symbol(p);
+        uint32_t v = reinterpret_cast<const Sym *>(inb)[p];
         if (is_ptr) {
           const uint32_t x = info[p];
           v = (x & 0xFFu) | (((x >> 8) - 1) << 8);
@@ -206,7 +274,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
         }
       }
       if (threadIdx.x < tail) pay[pb - tail + threadIdx.x] = inb[k * S + threadIdx.x];
-    } else {
+    } else if (stored) {
       ntok = 0;
       fb = 0;
       pb = bytes;
@@ -225,7 +293,7 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     __syncthreads();
     if (uint8_t *o = s_out) {
       if (warp == 0 && fb) warp_copy(o, reinterpret_cast<const uint8_t *>(flags), fb, lane);
-      const uint8_t *from = stored ? inb : pay;
+      const uint8_t *from = stored || literal ? inb : pay;
       const uint32_t part = (pb / kCoopWarps + 16) & ~15u;
       const uint32_t at = min(pb, warp * part), n = min(pb - at, part);
       if (n) warp_copy(o + fb + at, from + at, n, lane);
