@@ -139,7 +139,7 @@ class ClockSampler:
 # The compression kernel's sources: a DRAM traffic figure from an ncu capture
 # holds only while these are unchanged.
 KERNEL_SOURCES = ("compress_impl.cuh", "compress_launch.cuh", "compress_s4.cu",
-                  "glz_common.h", "glz_device.cuh")
+                  "glz_common.h", "glz_device.cuh", "mask_parse.cuh")
 PROFILE = os.path.join(ROOT, "profiles", "compress_kernel_field-256MiB.md")
 
 

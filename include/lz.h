@@ -243,13 +243,16 @@ lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes, const lz_param
                               void *d_out, uint64_t out_cap, uint64_t *d_out_bytes,
                               lz_stream_t stream);
 
-/* ---- Batches: many buffers in one persistent launch ------------------------
+/* ---- Batches: many buffers in a few persistent launches ---------------------
  * A batch is planned once on the host (lz_batch_create: validates every item,
  * uploads per-buffer descriptors, sizes and allocates its own scratch) and
- * run any number of times (lz_batch_run: a scratch clear and one persistent
- * kernel whose warps take chunks of all buffers from one work counter; no
- * host synchronisation, no allocation, so a run can be captured in a CUDA
- * graph and replayed).  The result of every item is byte-identical to
+ * run any number of times (lz_batch_run: decompression is one persistent
+ * kernel over the chunks of all streams; compression is a scratch clear and
+ * one kernel per class of buffers -- symbol size, parse, range of windows --
+ * whose warps take chunks from the class's work counter, the classes side by
+ * side on streams of the batch that start after what the caller's stream
+ * holds and that the caller's stream waits for; no host synchronisation, no
+ * allocation, so a run can be captured in a CUDA graph and replayed).  The result of every item is byte-identical to
  * lz_compress / lz_decompress of that item alone.  Device errors are sticky
  * in the context, as for the single-buffer calls. */
 typedef struct lz_batch_item {
@@ -450,8 +453,8 @@ uint64_t lz_huff_bound(uint64_t n_bytes);
 
 /* Huffman-code n_bytes at d_in (any alignment) into d_out (8-byte aligned,
  * capacity out_cap) and store the stream size in *d_out_bytes (device
- * uint64, 8-byte aligned).  Five launches (histogram, code book, sub-block
- * sizes, block offsets, encode); no host synchronisation.  out_cap below
+ * uint64, 8-byte aligned).  Three launches (histogram, code book, encode);
+ * no host synchronisation.  out_cap below
  * the header and tables is LZ_ERR_BUFFER_TOO_SMALL at once; a stream that
  * does not fit is reported by lz_sync (LZ_ERR_BUFFER_TOO_SMALL) with the
  * size that was needed in *d_out_bytes.  lz_huff_bound(n_bytes) always

@@ -1,4 +1,4 @@
-"""Batched compression of many uneven buffers (one persistent launch).
+"""Batched compression of many uneven buffers (a few persistent launches).
 
 Builds the many-buffer workload (sizes log-uniform over [4 KiB, 16 MiB],
 element types drawn uniformly from 1-byte codes, 2-byte codes, float32
@@ -140,7 +140,7 @@ def time_gpu(torch, fn, steps: int, warmup: int = 3) -> float:
 
 
 def run(torch, codec, w: Workload, steps: int = 3, check: int = 64) -> dict:
-    """Batched (one persistent launch, CUDA graph) vs one plain launch per
+    """Batched (persistent launches, CUDA graph) vs one plain launch per
     buffer, for compression and decompression of the whole workload."""
     stream = torch.cuda.current_stream()
     items = compress_items(w)
@@ -225,7 +225,10 @@ def run(torch, codec, w: Workload, steps: int = 3, check: int = 64) -> dict:
         "decompress_per_buffer_gbs": round(n / t_dplain / 1e9, 3),
         "ratio": round(n / float(sizes.sum()), 4),
         "sizes_equal_per_buffer": bool(same),
-        "launches": {"batched": 2, "per_buffer": 2 * len(items)},
+        # compression: one launch per class (symbol size and range of windows)
+        "launches": {"batched": 1 + len({(p.S, max(128, 1 << (p.W - 1).bit_length()))
+                                         for p in w.params}),
+                     "per_buffer": 2 * len(items)},
         "graphs": "both batched runs replayed from captured CUDA graphs",
         "params": [dict(kind=KIND_NAMES[k], S=p.S, C=p.C, W=p.W, m=p.m, M=p.M)
                    for k, p in enumerate(w.params)],
