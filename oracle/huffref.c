@@ -258,7 +258,7 @@ int huffref_decompress(const uint8_t *in, uint64_t in_bytes, uint8_t *out,
     uint64_t end = h_get_u64(in + table_at + 8u * b);
     if (end < pos - bits_at) return H_ECORRUPT;
     uint64_t bytes = end - (pos - bits_at);
-    if (bytes % 4 || pos + bytes > in_bytes) return H_ECORRUPT;
+    if (bytes % 4 || bytes > in_bytes - pos) return H_ECORRUPT;
     const uint8_t *blk = in + pos;
     uint64_t lo = b * HUFFREF_BLOCK;
     uint64_t hi = lo + HUFFREF_BLOCK < n ? lo + HUFFREF_BLOCK : n;

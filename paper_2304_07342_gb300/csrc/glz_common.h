@@ -27,6 +27,16 @@ constexpr uint32_t kErrInternal = 1u << 3;  // a device consistency check failed
 // raises kErrTimeout instead of hanging the GPU.
 constexpr uint32_t kSpinLimit = 1u << 22;
 
+// Does a block of a GHF1 stream of `in_bytes` bytes, whose table says that it
+// spans [start, end) of the bits at `bits_at` (<= in_bytes), lie inside the
+// stream, as a whole number of words?  No sum is formed of values that come
+// from the table (an end near 2^64 would wrap it past the check).
+__host__ __device__ inline bool huf_span_ok(uint64_t start, uint64_t end, uint64_t bits_at,
+                                            uint64_t in_bytes) {
+  return start <= end && end <= in_bytes - bits_at && (end - start) % 4 == 0 &&
+         end - start <= (1ull << 20);
+}
+
 // The parse by equality masks (mask_parse.cuh) takes the exact matchers when
 // records can be written over the staged chunk (S * m >= 1 + offB), the first
 // m rows of any position lie in the two slabs kept (m <= 32) and the window

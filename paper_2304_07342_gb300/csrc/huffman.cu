@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(256) huff_decode_kernel(const uint8_t *in, uin
     const uint64_t start = b ? ld_u64_le(table + 8 * (b - 1)) : 0ull;
     const uint64_t end = ld_u64_le(table + 8 * b);
     const uint64_t bytes = end - start;
-    bool bad = end < start || bytes % 4 || h.bits_at + end > in_bytes || bytes > (1ull << 20);
+    bool bad = !huf_span_ok(start, end, h.bits_at, in_bytes);
     const uint32_t nbits = static_cast<uint32_t>(bytes * 8);
     uint64_t lo, hi;
     sub_range(b, lane, h.n, lo, hi);
