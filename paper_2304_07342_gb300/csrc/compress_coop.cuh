@@ -148,15 +148,22 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     bool staged = true;
     if (bulk) {
       staged = mbar_wait_bounded(&bar, phase, A.spin_limit);
+      // a copy given up may still write the chunk: it is waited for (bounded
+      // again) before the block moves on to leave
+      if (!staged) mbar_wait_bounded(&bar, phase);
       phase ^= 1u;
     }
     staged = __syncthreads_and(staged);
     if (!staged && threadIdx.x == 0) atomicOr(A.err, kErrTimeout);
 
-    // (tried after a chunk without pointers, as with one warp per chunk; the
-    // filter takes the place of `info`)
-    const bool literal = try_literal && literal_chunk_block<S>(
-        reinterpret_cast<const Sym *>(inb), k, B, info, 32 * nslab, s_flagged, &s_count, warp, lane);
+    // A chunk that was not staged is not parsed (its symbols may change under
+    // the parse): it is published as literals and nothing of it is placed.
+    // (The pre-check is tried after a chunk without pointers, as with one warp
+    // per chunk; the filter takes the place of `info`.)
+    const bool literal =
+        !staged ||
+        (try_literal && literal_chunk_block<S>(reinterpret_cast<const Sym *>(inb), k, B, info,
+                                               32 * nslab, s_flagged, &s_count, warp, lane));
     const bool overlap = B.match == kMatchOverlap;
     const uint32_t m = B.m, M = B.M, W = B.W, tsz = 1 + B.offB;
     const uint32_t r = 31 - lane;
@@ -212,6 +219,14 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
             const uint32_t q = 32 * s + 31 - (__ffs(tok) - 1);
             uint32_t l, d;
             window_match<S, NW>(reinterpret_cast<const Sym *>(inb), k, B, q, lane, l, d);
+            // (the match is at least as long as the rows showed: the parse
+            // always moves on)
+            if (l < (info[q] & 0xFFu)) {
+              if (lane == 0) atomicOr(A.err, kErrInternal);
+              l = info[q] & 0xFFu;
+              d = info[q] >> 8;
+            }
+            __syncwarp();
             if (lane == 0) info[q] = l | (d << 8);
             next = q + l;
           }

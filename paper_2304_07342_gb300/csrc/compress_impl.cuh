@@ -1023,8 +1023,11 @@ __device__ __forceinline__ bool compress_chunk(const CompressArgs &A, const BufD
   bool staged = true;
   if (bulk) {
     staged = mbar_wait_bounded(W.bar, W.phase, A.spin_limit);
+    if (!staged) {
+      if (lane == 0) atomicOr(A.err, kErrTimeout);
+      mbar_wait_bounded(W.bar, W.phase);  // as in compress_coop.cuh
+    }
     W.phase ^= 1u;
-    if (!staged && lane == 0) atomicOr(A.err, kErrTimeout);
   }
   __syncwarp();
 
@@ -1035,11 +1038,12 @@ __device__ __forceinline__ bool compress_chunk(const CompressArgs &A, const BufD
   // check mostly gives up), else the candidate filter (hash table in the
   // payload area)
   const uint32_t bm_words = (A.sm.maybe_off - A.sm.prev_off) / 4;
-  bool literal = false;
+  // (a chunk that was not staged is not parsed: its symbols may still change)
+  bool literal = !staged;
   // (tried when this warp's previous chunk was all literals: on data with
   // repeats the check would only give up, so it is not tried again until a
   // chunk without a match comes by)
-  if (S >= 2 && W.try_literal && bm_words >= 16 && 4 * bm_words >= k)
+  if (S >= 2 && staged && W.try_literal && bm_words >= 16 && 4 * bm_words >= k)
     literal = literal_chunk<S>(sym, k, B, reinterpret_cast<uint32_t *>(W.links_base), bm_words,
                                W.maybe, lane);
   // 3. greedy parse.  By masks: the record itself, in shared memory.  By
