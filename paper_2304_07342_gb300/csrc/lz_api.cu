@@ -282,7 +282,7 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
                           uint32_t match, uint32_t version, void *d_out, uint64_t out_cap,
                           unsigned long long *out_bytes, cudaStream_t st, uint64_t c0 = 0,
                           uint64_t c1 = ~0ull, bool clear_status = true,
-                          uint32_t warps_per_block = 0);
+                          uint32_t warps_per_block = 0, bool block_per_chunk = true);
 
 }  // namespace
 
@@ -428,7 +428,8 @@ namespace {
 lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const lz_params *p,
                           uint32_t match, uint32_t version, void *d_out, uint64_t out_cap,
                           unsigned long long *out_bytes, cudaStream_t st, uint64_t c0,
-                          uint64_t c1, bool clear_status, uint32_t warps_per_block) {
+                          uint64_t c1, bool clear_status, uint32_t warps_per_block,
+                          bool block_per_chunk) {
   const uint32_t S = p->symbol_bytes, C = p->chunk_bytes;
   const uint64_t nc = div_up(n_bytes, C);
   if (c1 > nc) c1 = nc;
@@ -499,9 +500,9 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
   A.end_chunk = static_cast<uint32_t>(c1);
   uint32_t nj = 1;
   while (32 * nj < p->window) nj *= 2;
-  // (a caller's launch shape and the pieces of lz_compress_host keep one warp
-  // per chunk)
-  if (!warps_per_block && c0 == 0 && c1 == nc &&
+  // (a caller's launch shape, the pieces of lz_compress_host and the trials of
+  // the autotuner keep one warp per chunk)
+  if (block_per_chunk && !warps_per_block && c0 == 0 && c1 == nc &&
       glz::mask_parse_takes(S, p->window, p->min_match, A.buf.match) &&
       coop_takes(ctx, nc, wpb * best_blocks * ctx->sms, S, C, std::max(nj, 4u), &A.coop))
     return cuda_status(launch_coop(A, S, std::max(nj, 4u), static_cast<unsigned>(nc), st));
@@ -1527,14 +1528,19 @@ lz_status lz_autotune_ex(lz_ctx *ctx, const void *d_sample, uint64_t sample_byte
       cudaEventCreate(&e1) != cudaSuccess)
     s = LZ_ERR_NOMEM;
   // one trial: three compressions (the first warms up), the mean of the
-  // last two, and the ratio
+  // last two, and the ratio.  Always with one warp per chunk: the sample
+  // stands for buffers of any size, and its own would choose between that
+  // and a block per chunk differently for every chunk size.
   auto run = [&](lz_tune_trial &t) {
-    lz_options opt{LZ_MATCH_EXACT, 1, t.warps_per_block};
     t.seconds = 0;
     for (int rep = 0; rep < 3 && s == LZ_OK; ++rep) {
       cudaEventRecord(e0, nullptr);
-      s = lz_compress_ex(ctx, d_sample, sample_bytes, &t.params, &opt, d_out, cap,
-                         static_cast<uint64_t *>(d_nb), nullptr);
+      {
+        std::lock_guard<std::mutex> lock(ctx->mu);
+        s = compress_locked(ctx, d_sample, sample_bytes, &t.params, LZ_MATCH_EXACT, 1, d_out, cap,
+                            static_cast<unsigned long long *>(d_nb), nullptr, 0, ~0ull, true,
+                            t.warps_per_block, false);
+      }
       cudaEventRecord(e1, nullptr);
       if (s == LZ_OK) s = lz_sync(ctx, nullptr);
       float ms = 0;
