@@ -115,6 +115,34 @@ __device__ __forceinline__ uint32_t lowest_bit(const uint32_t (&v)[NW]) {
   return at + __ffs(w);
 }
 
+// The bits in which the k symbols of a staged chunk differ, as Gray codes (one
+// warp).
+template <int S>
+__device__ __forceinline__ uint32_t varying_bits(const uint8_t *inb, uint32_t k, uint32_t lane) {
+  using Sym = typename SymType<S>::T;
+  constexpr uint32_t kBelow = S == 1 ? 0x7F7F7F7Fu : S == 2 ? 0x7FFF7FFFu : 0x7FFFFFFFu;
+  auto gray = [](uint32_t v) { return v ^ ((v >> 1) & kBelow); };  // of every symbol in v
+  const uint32_t first = reinterpret_cast<const Sym *>(inb)[0];
+  const uint32_t g0 = gray(S == 1 ? first * 0x01010101u : S == 2 ? first * 0x00010001u : first);
+  const uint32_t words = k * S / 4, quads = words / 4;  // whole words of symbols
+  uint32_t d = 0;
+#pragma unroll 1
+  for (uint32_t i = lane; i < quads; i += 32) {
+    const uint4 v = reinterpret_cast<const uint4 *>(inb)[i];
+    d |= (gray(v.x) ^ g0) | (gray(v.y) ^ g0) | (gray(v.z) ^ g0) | (gray(v.w) ^ g0);
+  }
+  if (lane < words - 4 * quads)
+    d |= gray(reinterpret_cast<const uint32_t *>(inb)[4 * quads + lane]) ^ g0;
+  if constexpr (S < 4) {
+    const uint32_t p = words * (4 / S) + lane;  // symbols after the last whole word
+    const uint32_t one = S == 1 ? 0xFFu : 0xFFFFu;
+    if (p < k) d |= (gray(reinterpret_cast<const Sym *>(inb)[p]) ^ g0) & one;
+  }
+  if constexpr (S == 1) d |= d >> 16, d |= d >> 8, d &= 0xFFu;
+  if constexpr (S == 2) d |= d >> 16, d &= 0xFFFFu;
+  return __reduce_or_sync(kFull, d);
+}
+
 // WHOLE: planes of every slab of the chunk are kept, else of the last 2 * NW.
 // COUNT: slabs made at a time; two share the plane words of the slabs before
 // them and the work around them (windows of 512 keep one: four slabs of their
@@ -143,29 +171,8 @@ struct MaskParser {
     return p < k ? static_cast<uint32_t>(reinterpret_cast<const Sym *>(inb)[p]) : 0u;
   }
 
-  // The bits in which the chunk's symbols differ, as Gray codes.
   __device__ __forceinline__ void find_varying_bits() {
-    constexpr uint32_t kBelow = S == 1 ? 0x7F7F7F7Fu : S == 2 ? 0x7FFF7FFFu : 0x7FFFFFFFu;
-    auto gray = [](uint32_t v) { return v ^ ((v >> 1) & kBelow); };  // of every symbol in v
-    const uint32_t first = reinterpret_cast<const Sym *>(inb)[0];
-    const uint32_t g0 = gray(S == 1 ? first * 0x01010101u : S == 2 ? first * 0x00010001u : first);
-    const uint32_t words = k * S / 4, quads = words / 4;  // whole words of symbols
-    uint32_t d = 0;
-#pragma unroll 1
-    for (uint32_t i = lane; i < quads; i += 32) {
-      const uint4 v = reinterpret_cast<const uint4 *>(inb)[i];
-      d |= (gray(v.x) ^ g0) | (gray(v.y) ^ g0) | (gray(v.z) ^ g0) | (gray(v.w) ^ g0);
-    }
-    if (lane < words - 4 * quads)
-      d |= gray(reinterpret_cast<const uint32_t *>(inb)[4 * quads + lane]) ^ g0;
-    if constexpr (S < 4) {
-      const uint32_t p = words * (4 / S) + lane;  // symbols after the last whole word
-      const uint32_t one = S == 1 ? 0xFFu : 0xFFFFu;
-      if (p < k) d |= (gray(symbol(p)) ^ g0) & one;
-    }
-    if constexpr (S == 1) d |= d >> 16, d |= d >> 8, d &= 0xFFu;
-    if constexpr (S == 2) d |= d >> 16, d &= 0xFFFFu;
-    act = __reduce_or_sync(kFull, d);
+    act = varying_bits<S>(inb, k, lane);
     ngroups = (__popc(act) + 7) / 8;
     uint32_t rest = act;
     next_lifts(rest, lift0);
@@ -298,6 +305,11 @@ struct MaskParser {
         e[j + 3] = t.w;
       }
     }
+  }
+  // Word j of E(p).
+  __device__ __forceinline__ uint32_t row_word(uint32_t p, uint32_t j) const {
+    const uint32_t at = (p & (kRows - 1)) * kPart;
+    return rows[NW <= 4 ? at + j : at + (j & ~3u) * kRows + (j & 3u)];
   }
   __device__ __forceinline__ void set_row(uint32_t p, const uint32_t (&e)[NW]) const {
     uint32_t *at = rows + (p & (kRows - 1)) * kPart;
@@ -448,32 +460,36 @@ __device__ __forceinline__ void mask_parse(uint8_t *inb, uint32_t k, uint32_t ta
       made += P.COUNT;
     }
     if (long_p != kNone) {
-      // the open match, through the rows of slabs s and s + 1
+      // the open match, through the rows of slabs s and s + 1: lane j < NW
+      // holds word j of its offsets (each lane holding all words took a
+      // hundred instructions a symbol at 16 words: 32 MiB of zero words,
+      // W = 512, 2,780 us, 758 so)
       const uint32_t lim = min(M, k - long_p), stop = min(lim, 32 * made - long_p);
-      uint32_t b[NW];
-      load_row<NW>(rows + P.kRows * NW, b);
+      const uint32_t word = min(lane, static_cast<uint32_t>(NW - 1));
+      uint32_t b = lane < NW ? rows[P.kRows * NW + word] : 0u;
       bool more = true;
 #pragma unroll 1
       while (long_len < stop) {
-        uint32_t e[NW];
-        P.row(long_p + long_len, e);
-        drop_offsets<NW>(e, overlap ? 0u : long_len);
-#pragma unroll
-        for (int j = 0; j < NW; ++j) e[j] &= b[j];
-        more = any_bit<NW>(e);
+        uint32_t e = P.row_word(long_p + long_len, word) & b;
+        if (!overlap) {  // offsets up to the length drop out
+          const uint32_t gone = long_len > 32 * word ? min(long_len - 32 * word, 32u) : 0u;
+          e &= __funnelshift_lc(0u, kFull, gone);
+        }
+        more = __any_sync(kFull, e != 0);
         if (!more) break;
-#pragma unroll
-        for (int j = 0; j < NW; ++j) b[j] = e[j];
+        b = e;
         ++long_len;
       }
       cur = long_p + long_len;
       if (more && long_len < lim) {  // still open
         __syncwarp();
-        if (lane == 0) store_row<NW>(rows + P.kRows * NW, b);
+        if (lane < NW) rows[P.kRows * NW + word] = b;
         __syncwarp();
         continue;
       }
-      const uint32_t v = long_len | ((lowest_bit<NW>(b) - 1) << 8);
+      const uint32_t at = __ffs(__ballot_sync(kFull, b != 0)) - 1;
+      const uint32_t low = 32 * at + __ffs(__shfl_sync(kFull, b, at));  // its nearest offset
+      const uint32_t v = long_len | ((low - 1) << 8);
       if (lane < tsz && GLZ_OK(long_at + lane < S * k))
         inb[long_at + lane] = static_cast<uint8_t>(v >> (8 * lane));
       long_p = kNone;
