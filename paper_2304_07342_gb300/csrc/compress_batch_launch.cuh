@@ -18,16 +18,25 @@ static cudaError_t launch_batch_nj(const CompressArgs &A, int block, unsigned gr
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const uint64_t cap = static_cast<uint64_t>(per_sm) * sms;
   const unsigned grid = static_cast<unsigned>(grid_req < cap ? grid_req : cap);
+  if (A.votes) return launch_dependent(kern, grid, block, smem, stream, A);
   kern<<<grid, block, smem, stream>>>(A);
   return cudaGetLastError();
 }
 
 // One class of a batch: windows of at most 32 * nj symbols.  A mask word
 // costs every position, so the mask parse has an instance for each class of
-// windows; the chains only need one- or two-byte links.
+// windows; the chains only need one- or two-byte links, and an instance for
+// each class where a sample chooses between the two.
 template <int S>
 static cudaError_t launch_batch_t(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                   unsigned grid, cudaStream_t stream) {
+  if (!mask && A.votes) {
+    switch (nj) {
+      case 4: return launch_batch_nj<S, 4, false>(A, block, grid, stream);
+      case 8: return launch_batch_nj<S, 8, false>(A, block, grid, stream);
+      default: return launch_batch_nj<S, 16, false>(A, block, grid, stream);
+    }
+  }
   if (!mask) {
     return nj <= 8 ? launch_batch_nj<S, 8, false>(A, block, grid, stream)
                    : launch_batch_nj<S, 32, false>(A, block, grid, stream);

@@ -260,6 +260,14 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
     try_literal = np == 0;
     uint32_t pb = S * (ntok - np) + tsz * np + tail, fb = (ntok + 7) / 8;
     const bool stored = B.version == 2 && fb + pb >= bytes;  // the chunk as it is
+    if (stored) {
+      ntok = 0;
+      fb = 0;
+      pb = bytes;
+    }
+    const uint64_t rec = static_cast<uint64_t>(fb) + pb;
+    // (published before the record is written, so that later chunks wait less)
+    if (c != 0 && warp == 0) publish(A.status + B.gbase, c, kAgg, rec, lane);
     if (!stored && !literal) {
       const uint32_t earlier = lane == 31 ? 0u : kFull << (lane + 1);
       for (uint32_t s = warp; s < nslab; s += kCoopWarps) {
@@ -289,14 +297,8 @@ __global__ void __launch_bounds__(32 * kCoopWarps, NW <= 8 ? 3 : 2)
         }
       }
       if (threadIdx.x < tail) pay[pb - tail + threadIdx.x] = inb[k * S + threadIdx.x];
-    } else if (stored) {
-      ntok = 0;
-      fb = 0;
-      pb = bytes;
     }
-    const uint64_t rec = static_cast<uint64_t>(fb) + pb;
     if (warp == 0) {
-      if (c != 0) publish(A.status + B.gbase, c, kAgg, rec, lane);
       uint8_t *tab = B.out + kHeaderBytes + static_cast<uint64_t>(kTableEntry) * c;
       if (lane < 4) tab[lane] = static_cast<uint8_t>(ntok >> (8 * lane));
       else if (lane < 8) tab[lane] = static_cast<uint8_t>(pb >> (8 * (lane - 4)));

@@ -7,4 +7,7 @@ cudaError_t launch_coop_s2(const CompressArgs &A, uint32_t nw, unsigned grid,
                            cudaStream_t stream) {
   return launch_coop_t<2>(A, nw, grid, stream);
 }
+cudaError_t coop_blocks_s2(uint32_t nw, uint32_t smem, int *per_sm) {
+  return coop_blocks_t<2>(nw, smem, per_sm);
+}
 }  // namespace glz

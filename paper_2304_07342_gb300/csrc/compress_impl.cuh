@@ -9,8 +9,8 @@
 //      filter over symbol keys, tried after a chunk without pointers;
 //      chunks without repeats end here as all literals).  Exact matchers with
 //      windows up to 512 then take the parse by equality masks
-//      (mask_parse.cuh), which does step 3 and the record as well; the
-//      others link every position to the last earlier position with the same hash of its
+//      (mask_parse.cuh), which does step 3 and the record as well, unless a
+//      sample says that the data seldom repeat (sample.cuh); the others link every position to the last earlier position with the same hash of its
 //      first min(m, 8/S) symbols (hash chains; __match_any_sync links
 //      positions of one 32-position slab) and marks the positions whose
 //      chain holds their key inside the window -- only those can start a
@@ -39,6 +39,7 @@
 #include "glz_common.h"
 #include "glz_device.cuh"
 #include "mask_parse.cuh"
+#include "sample.cuh"
 
 namespace glz {
 
@@ -226,7 +227,7 @@ __device__ __forceinline__ void build_chains(const typename SymType<S>::T *sym,
 // then p and q share the key: q is flagged (and (i) finds it) unless p and q
 // lie in one slab and p came second, in which case p is flagged and (ii)
 // finds it.
-constexpr uint32_t kBloomMaxFlagged = 16;
+constexpr uint32_t kBloomMaxFlagged = 16;  // at least: half a position per slab
 constexpr uint32_t kBloomGroup = 8;  // slabs whose ORs are issued together
 
 // Does p (flagged, p + m <= k) take part in a match of >= m symbols, as the
@@ -280,6 +281,7 @@ __device__ __forceinline__ bool literal_chunk(const typename SymType<S>::T *sym,
   const uint32_t mlo = kb >= 4 ? kFull : (1u << (8 * kb)) - 1u;
   const uint32_t mhi = kb <= 4 ? 0u : (kb >= 8 ? kFull : (1u << (8 * (kb - 4))) - 1u);
   const uint32_t nslab = (k + 31) / 32;
+  const uint32_t max_flagged = max(kBloomMaxFlagged, nslab / 2);
   uint32_t nflag = 0;
   // groups of kBloomGroup slabs: keys and masks first, then the ORs in slab
   // order (each behind the previous one), then the votes, so that the ORs of
@@ -311,7 +313,7 @@ __device__ __forceinline__ bool literal_chunk(const typename SymType<S>::T *sym,
       if (lane == 0 && s0 + u < nslab) maybe[s0 + u] = f;
       nflag += __popc(f);
     }
-    if (nflag > kBloomMaxFlagged) return false;
+    if (nflag > max_flagged) return false;
   }
   __syncwarp();
   if (nflag == 0) return true;
@@ -1179,17 +1181,36 @@ __device__ __forceinline__ uint32_t take_ticket(const CompressArgs &A, uint32_t 
 // the shared memory would keep resident; the limits are what the register
 // file gives the warps that fit: 72 at windows up to 128 (28 warps per SM at
 // S = 2, C = 4096: 2,140 us for 256 MiB of quantization codes, 2,230 at 64
-// with spills, 2,185 at 80), 96 up to 256 (21 warps at S = 4, C = 4096: 860 us
-// for 128 MiB of Markov words, 925 at 80, 936 at 104), 128 up to 512 (15 warps
-// at S = 1, C = 8192).
-constexpr int reg_limit(int nj, bool mask) {
-  return mask ? (nj <= 4 ? 72 : nj <= 8 ? 96 : 128) : (nj < 32 ? 64 : 80);
+// with spills, 2,185 at 80), 96 up to 256 (20 warps at S = 4, C = 4096: 860 us
+// for 128 MiB of Markov words, 925 at 80, 936 at 104), 128 up to 512 (14 warps
+// at S = 1, C = 8192).  The chains can do with 64 but take what their slices
+// leave (256 MiB of a float field, all literals: 205 us at 64, 198 at 96).
+constexpr int reg_limit(int S, int nj, bool mask) {
+  if (mask) return nj <= 4 ? 72 : nj <= 8 ? 96 : 128;
+  return nj <= 4 ? 72 : nj <= 8 && S < 4 ? 80 : 96;
+}
+
+// Masks and chains are launched one after the other when a sample of the data
+// chooses between them (A.votes, sample.cuh); the one that it did not choose
+// ends here.  (With both parses in one kernel, whichever way they were kept
+// apart, the masks took 3 to 12 % longer: 4-byte codes, W = 256, 608 to 716
+// instructions a slab, 596 alone.)
+template <int S, int NJ, bool MASK>
+__device__ __forceinline__ bool chosen(const CompressArgs &A) {
+  if constexpr (32 * NJ <= kMaskMaxWindow) {
+    if (A.votes) {
+      grid_wait();
+      return seldom_repeats<S, NJ>(A.votes) != MASK;
+    }
+  }
+  return true;
 }
 
 // Single buffer: the symbol size is a template parameter.
 template <int S, int NJ, bool MASK>
-__global__ void __maxnreg__(reg_limit(NJ, MASK)) compress_kernel(const CompressArgs A) {
+__global__ void __maxnreg__(reg_limit(S, NJ, MASK)) compress_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
+  if (!chosen<S, NJ, MASK>(A)) return;
   const uint32_t lane = threadIdx.x & 31;
   WarpState W;
   init_warp_state(A, smem, W, lane);
@@ -1224,9 +1245,10 @@ __device__ __forceinline__ uint32_t find_item(const CompressArgs &A, uint64_t g,
 // size, parse and range of windows) in order; each buffer carries its own
 // parameters, kept in shared memory while one of its chunks is compressed.
 template <int S, int NJ, bool MASK>
-__global__ void __maxnreg__(reg_limit(NJ, MASK)) compress_batch_kernel(const CompressArgs A) {
+__global__ void __maxnreg__(reg_limit(S, NJ, MASK)) compress_batch_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
   __shared__ BufDesc descs[8];
+  if (!chosen<S, NJ, MASK>(A)) return;
   const uint32_t lane = threadIdx.x & 31;
   BufDesc &B = descs[threadIdx.x >> 5];
   WarpState W;

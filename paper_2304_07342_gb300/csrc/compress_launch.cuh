@@ -23,29 +23,29 @@ static cudaError_t launch_compress_nj(const CompressArgs &A, int block, unsigned
   // more than the parking slots were sized for
   const uint64_t cap = static_cast<uint64_t>(per_sm) * sms;
   const unsigned grid = static_cast<unsigned>(grid_req < cap ? grid_req : cap);
+  if (A.votes) return launch_dependent(kern, grid, block, smem, stream, A);
   kern<<<grid, block, smem, stream>>>(A);
   return cudaGetLastError();
 }
 
 template <int S, int NJ>
-static cudaError_t launch_compress_mode(const CompressArgs &A, int block, unsigned grid,
+static cudaError_t launch_compress_mode(const CompressArgs &A, bool mask, int block, unsigned grid,
                                         cudaStream_t stream) {
   if constexpr (32 * NJ <= kMaskMaxWindow)
-    if (mask_parse_takes(S, A.buf.W, A.buf.m, A.buf.match))
-      return launch_compress_nj<S, NJ, true>(A, block, grid, stream);
+    if (mask) return launch_compress_nj<S, NJ, true>(A, block, grid, stream);
   return launch_compress_nj<S, NJ, false>(A, block, grid, stream);
 }
 
 template <int S>
-static cudaError_t launch_compress_t(const CompressArgs &A, uint32_t nj,
+static cudaError_t launch_compress_t(const CompressArgs &A, uint32_t nj, bool mask,
                                      int block, unsigned grid, cudaStream_t stream) {
   switch (nj) {
-    case 1: return launch_compress_mode<S, 1>(A, block, grid, stream);
-    case 2: return launch_compress_mode<S, 2>(A, block, grid, stream);
-    case 4: return launch_compress_mode<S, 4>(A, block, grid, stream);
-    case 8: return launch_compress_mode<S, 8>(A, block, grid, stream);
-    case 16: return launch_compress_mode<S, 16>(A, block, grid, stream);
-    case 32: return launch_compress_mode<S, 32>(A, block, grid, stream);
+    case 1: return launch_compress_mode<S, 1>(A, mask, block, grid, stream);
+    case 2: return launch_compress_mode<S, 2>(A, mask, block, grid, stream);
+    case 4: return launch_compress_mode<S, 4>(A, mask, block, grid, stream);
+    case 8: return launch_compress_mode<S, 8>(A, mask, block, grid, stream);
+    case 16: return launch_compress_mode<S, 16>(A, mask, block, grid, stream);
+    case 32: return launch_compress_mode<S, 32>(A, mask, block, grid, stream);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -1,11 +1,16 @@
-// compress_s1.cu -- instantiations of the compression kernel for
+// compress_s1.cu -- instantiations of the compression and sampling kernels for
 // 1-byte symbols (one translation unit per symbol size so that the
 // variants compile in parallel).
 #include "compress_launch.cuh"
+#include "sample_launch.cuh"
 
 namespace glz {
-cudaError_t launch_compress_s1(const CompressArgs &A, uint32_t nj, int block,
+cudaError_t launch_compress_s1(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                unsigned grid, cudaStream_t stream) {
-  return launch_compress_t<1>(A, nj, block, grid, stream);
+  return launch_compress_t<1>(A, nj, mask, block, grid, stream);
+}
+cudaError_t launch_sample_s1(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
+                             cudaStream_t stream) {
+  return launch_sample_t<1>(A, nj, clear, clear_bytes, stream);
 }
 }  // namespace glz

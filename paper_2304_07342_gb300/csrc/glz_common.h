@@ -61,6 +61,9 @@ __host__ __device__ constexpr uint32_t mask_rows_bytes(uint32_t nw, uint32_t mad
   return ((64 * made + 1) * nw * 4 + 15) & ~15u;
 }
 
+// The sample that chooses between masks and chains: one word per sampling warp.
+constexpr uint32_t kSampleWarps = 64;
+
 // Per-warp shared-memory layout of the compressor (byte offsets from the
 // warp's slice; every region 16-byte aligned).
 struct CompressSmem {
@@ -140,6 +143,8 @@ struct CompressArgs {
   CoopSmem coop;               // or the layout of a block per chunk
   unsigned long long *status;  // one look-back word per chunk (cleared per call)
   uint32_t *ticket;            // work counter (cleared per call)
+  uint32_t *votes;             // kSampleWarps words, samples of the launch's data (sample.cuh);
+                               // null: this kernel takes the launch whatever its data
   uint32_t *err;               // sticky error bits
   uint8_t *park;               // parking slots: grid warps x park_slots
   uint32_t park_slots;         // slots per warp (<= 32)

@@ -100,6 +100,17 @@ __device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes) {
                : "memory");
 }
 
+// ---- programmatic dependent launch -------------------------------------------
+
+// Wait until the grid before this one on the stream has ended and its writes
+// are visible (nothing to wait for in an ordinary launch).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The next grid on the stream may be launched once every block has come here.
+__device__ __forceinline__ void grid_launch_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- relaxed device-scope status words -----------------------------------------
 
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long *p,

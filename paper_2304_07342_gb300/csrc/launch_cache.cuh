@@ -54,4 +54,23 @@ static cudaError_t resident_blocks(LaunchCache &lc, K kern, int block,
   return cudaSuccess;
 }
 
+// Launch that may begin while the kernel before it on the stream still runs
+// (programmatic dependent launch): the kernel waits for that one itself
+// (grid_wait) before it touches anything of it.
+template <typename K, typename... Args>
+static cudaError_t launch_dependent(K kern, unsigned grid, int block, size_t smem,
+                                    cudaStream_t stream, const Args &...args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
 }  // namespace glz

@@ -14,16 +14,25 @@
 #include "glz_common.h"
 
 namespace glz {
-cudaError_t launch_compress_s1(const CompressArgs &A, uint32_t nj, int block,
+cudaError_t launch_compress_s1(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                unsigned grid, cudaStream_t stream);
-cudaError_t launch_compress_s2(const CompressArgs &A, uint32_t nj, int block,
+cudaError_t launch_compress_s2(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                unsigned grid, cudaStream_t stream);
-cudaError_t launch_compress_s4(const CompressArgs &A, uint32_t nj, int block,
+cudaError_t launch_compress_s4(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                unsigned grid, cudaStream_t stream);
+cudaError_t launch_sample_s1(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
+                             cudaStream_t stream);
+cudaError_t launch_sample_s2(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
+                             cudaStream_t stream);
+cudaError_t launch_sample_s4(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
+                             cudaStream_t stream);
 cudaError_t launch_decompress(DecompressArgs A, int block, cudaStream_t stream);
 cudaError_t launch_coop_s1(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
 cudaError_t launch_coop_s2(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
 cudaError_t launch_coop_s4(const CompressArgs &A, uint32_t nw, unsigned grid, cudaStream_t stream);
+cudaError_t coop_blocks_s1(uint32_t nw, uint32_t smem, int *per_sm);
+cudaError_t coop_blocks_s2(uint32_t nw, uint32_t smem, int *per_sm);
+cudaError_t coop_blocks_s4(uint32_t nw, uint32_t smem, int *per_sm);
 cudaError_t launch_batch_empties(const BufDesc *empties, uint32_t n, cudaStream_t stream);
 cudaError_t launch_batch_class(const CompressArgs &A, uint32_t S, uint32_t nj, bool mask,
                                int block, unsigned grid, cudaStream_t stream);
@@ -100,6 +109,7 @@ constexpr int kCompressWarps = 4;      // warps per block (fewer if smem-bound)
 constexpr uint32_t kParkSlots = 3;     // parked records per compressing warp
 constexpr int kDecompressBlock = 1024;  // up to 32 warps, one chunk per warp at a time
 constexpr size_t kScratchHead = 16;
+constexpr size_t kSampleBytes = 4 * glz::kSampleWarps;
 // The look-back word of a placed chunk (written by the compression kernel):
 // bit 63 set, the inclusive prefix of the record bytes in the low 62 bits.
 constexpr uint64_t kStatusPrefix = 1ull << 63, kStatusValue = (1ull << 62) - 1;
@@ -113,6 +123,7 @@ constexpr uint64_t kMaxLaunchChunks = 0xFFFFFFFFull - (1ull << 20);
 
 uint64_t div_up(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 uint32_t round16(uint64_t v) { return static_cast<uint32_t>((v + 15) & ~15ull); }
+uint64_t round16_64(uint64_t v) { return (v + 15) & ~15ull; }
 uint32_t off_bytes(uint32_t W) { return W <= 256 ? 1u : 2u; }
 
 // Worst-case record of a chunk of k symbols (see lz_compressed_bound).
@@ -139,8 +150,9 @@ uint32_t kernel_match(uint32_t match) {
                                      : glz::kMatchExact;
 }
 
-// Shared-memory slice of one compressing warp (`match`: the kernels').
-glz::CompressSmem compress_layout(const lz_params *p, uint32_t match) {
+// Shared-memory slice of one compressing warp, with the parse by masks or by
+// chains.
+glz::CompressSmem compress_layout(const lz_params *p, bool masks) {
   const uint32_t S = p->symbol_bytes, C = p->chunk_bytes;
   const uint32_t k = C / S;
   const uint32_t offB = off_bytes(p->window);
@@ -169,7 +181,7 @@ glz::CompressSmem compress_layout(const lz_params *p, uint32_t match) {
     const uint64_t table = 2ull << lgt;
     pay_region = round16((list > table ? list : table) + 16);
   }
-  if (glz::mask_parse_takes(S, p->window, p->min_match, match)) {
+  if (masks) {
     // Bit planes in place of the links and rows in place of the payload area.
     // 1-byte symbols have no literal pre-check and take no more than these:
     // 14 KiB instead of 34 per warp at C = 8192, W = 512, 15 warps resident
@@ -177,7 +189,8 @@ glz::CompressSmem compress_layout(const lz_params *p, uint32_t match) {
     // one-byte links) for the pre-check's bitmap.
     uint32_t nw = 4;  // (a batch runs small windows with 4 words)
     while (32 * nw < p->window) nw *= 2;
-    const uint32_t planes = glz::mask_planes_bytes(S, nw), rows = glz::mask_rows_bytes(nw, glz::mask_slabs_made(nw));
+    const uint32_t planes = glz::mask_planes_bytes(S, nw);
+    const uint32_t rows = glz::mask_rows_bytes(nw, glz::mask_slabs_made(nw));
     const uint32_t kept = S == 1 ? 0u : round16(k) + pay_region;
     links = planes;
     pay_region = std::max(rows, kept > planes ? kept - planes : 0u);
@@ -224,16 +237,62 @@ bool block_shape(int64_t per_warp, int smem_per_sm, int smem_reserved, int smem_
   return best_warps > 0;
 }
 
+// The launch of one warp per chunk: the slice, the block and the blocks that a
+// multiprocessor holds.
+struct WarpShape {
+  glz::CompressSmem sm;
+  int block = 32;
+  int64_t blocks_per_sm = 0;  // 0: not even one fits
+
+  uint64_t warps() const { return block / 32; }
+  // Blocks for `chunks` chunks, at most what is resident.
+  uint64_t grid(uint64_t chunks, int sms) const {
+    return std::min(div_up(chunks, warps()), static_cast<uint64_t>(blocks_per_sm) * sms);
+  }
+};
+
+WarpShape warp_shape(const glz::CompressSmem &sm, int smem_per_sm, int smem_reserved,
+                     int smem_optin, uint32_t want) {
+  WarpShape w;
+  w.sm = sm;
+  if (static_cast<int64_t>(sm.per_warp) > smem_optin ||
+      !block_shape(sm.per_warp, smem_per_sm, smem_reserved, smem_optin, want, &w.block,
+                   &w.blocks_per_sm))
+    w.blocks_per_sm = 0;
+  return w;
+}
+
+// The chains beside a parse by masks, of whose launch shape `want` is: their
+// slice is larger, so they may need the library's own choice.
+WarpShape chains_shape(const glz::CompressSmem &sm, int smem_per_sm, int smem_reserved,
+                       int smem_optin, uint32_t want) {
+  WarpShape w = warp_shape(sm, smem_per_sm, smem_reserved, smem_optin, want);
+  if (!w.blocks_per_sm) w = warp_shape(sm, smem_per_sm, smem_reserved, smem_optin, 0);
+  return w;
+}
+
 // Does a launch over `chunks` chunks take a block of eight warps per chunk
-// (compress_coop.cuh)?  When they would fill less than half of the warps that
-// one warp per chunk keeps resident, and the block fits: below that line a
-// launch lasts as long as one chunk.  Gives the layout for chunks of C bytes
-// and windows of 32 * nw symbols.
-bool coop_takes(const lz_ctx *ctx, uint64_t chunks, uint64_t resident_warps, uint32_t S,
-                uint32_t C, uint32_t nw, glz::CoopSmem *out) {
-  if (2 * chunks > resident_warps) return false;
+// (compress_coop.cuh)?  When the blocks for all of them are resident at once,
+// or twice over: below that line a launch lasts about as long as one chunk,
+// beyond it a block's eight warps do less than eight warps with a chunk each
+// (2-byte codes, C = 4096, 456 blocks at once: 3 MiB 69 us by blocks, 91 by
+// warps, 8 MiB 148 and 117).  4-byte symbols, which more often hold few repeats
+// (chains, one warp per chunk), only once (W = 128, C = 4096, 2 MiB: codes 45
+// us by blocks, 57 by warps; few repeats 87 and 43).  Gives the layout for
+// chunks of C bytes and windows of 32 * nw symbols.
+uint64_t coop_waves(uint32_t S) { return S == 4 ? 1 : 2; }
+
+bool coop_takes(const lz_ctx *ctx, uint64_t chunks, uint32_t S, uint32_t C, uint32_t nw,
+                glz::CoopSmem *out) {
+  // (registers keep at most three blocks on an SM)
+  if (chunks > coop_waves(S) * 3 * ctx->sms || C / S > 0x7E00) return false;  // positions and a flag in 16 bits
   *out = glz::coop_layout(S, C, nw);
-  return static_cast<int64_t>(out->total) + 1024 <= ctx->smem_optin && C / S <= 0x7E00;  // positions and the flag in 16 bits
+  if (static_cast<int64_t>(out->total) + 1024 > ctx->smem_optin) return false;
+  int per_sm = 0;
+  const cudaError_t e = S == 1   ? glz::coop_blocks_s1(nw, out->total, &per_sm)
+                        : S == 2 ? glz::coop_blocks_s2(nw, out->total, &per_sm)
+                                 : glz::coop_blocks_s4(nw, out->total, &per_sm);
+  return e == cudaSuccess && chunks <= coop_waves(S) * per_sm * ctx->sms;
 }
 
 cudaError_t launch_coop(const glz::CompressArgs &A, uint32_t S, uint32_t nw, unsigned grid,
@@ -243,6 +302,35 @@ cudaError_t launch_coop(const glz::CompressArgs &A, uint32_t S, uint32_t nw, uns
     case 2: return glz::launch_coop_s2(A, nw, grid, st);
     default: return glz::launch_coop_s4(A, nw, grid, st);
   }
+}
+
+// The sample before a launch with the parse by masks (sample.cuh), which also
+// clears `clear_bytes` (a multiple of 16) at `clear`.
+cudaError_t launch_sample(const glz::CompressArgs &A, uint32_t S, uint32_t nj, void *clear,
+                          uint64_t clear_bytes, cudaStream_t st) {
+  switch (S) {
+    case 1: return glz::launch_sample_s1(A, nj, clear, clear_bytes, st);
+    case 2: return glz::launch_sample_s2(A, nj, clear, clear_bytes, st);
+    default: return glz::launch_sample_s4(A, nj, clear, clear_bytes, st);
+  }
+}
+
+// One warp per chunk over `chunks` chunks of one buffer: by masks (`mask`) or
+// chains in shape `w`, and by chains in shape `chains` where the data decide.
+cudaError_t launch_parses(glz::CompressArgs A, uint32_t nj, bool mask, const WarpShape &w,
+                          const WarpShape &chains, uint64_t chunks, int sms, cudaStream_t st) {
+  auto go = [&](bool by_masks, const WarpShape &x) {
+    A.sm = x.sm;
+    const unsigned grid = static_cast<unsigned>(x.grid(chunks, sms));
+    switch (A.buf.S) {
+      case 1: return glz::launch_compress_s1(A, nj, by_masks, x.block, grid, st);
+      case 2: return glz::launch_compress_s2(A, nj, by_masks, x.block, grid, st);
+      default: return glz::launch_compress_s4(A, nj, by_masks, x.block, grid, st);
+    }
+  };
+  cudaError_t e = A.votes ? go(false, chains) : cudaSuccess;
+  if (e == cudaSuccess) e = go(mask, w);
+  return e;
 }
 
 lz_status cuda_status(cudaError_t e) {
@@ -442,31 +530,30 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
                                           p->min_match, p->max_match, C,
                                           p->window, out_bytes, st));
 
-  glz::CompressSmem sm = compress_layout(p, kernel_match(match));
-  if (static_cast<int64_t>(sm.per_warp) > ctx->smem_optin) return LZ_ERR_INVALID_ARG;
-  int block = 32;
-  int64_t best_blocks = 1;
-  if (!block_shape(sm.per_warp, ctx->smem_per_sm, ctx->smem_reserved, ctx->smem_optin,
-                   warps_per_block, &block, &best_blocks))
-    return LZ_ERR_INVALID_ARG;
-  const uint64_t wpb = block / 32;
-  uint64_t grid = div_up(c1 - c0, wpb);
-  if (grid > static_cast<uint64_t>(best_blocks) * ctx->sms) grid = best_blocks * ctx->sms;
+  const bool mask = glz::mask_parse_takes(S, p->window, p->min_match, kernel_match(match));
+  const WarpShape w = warp_shape(compress_layout(p, mask), ctx->smem_per_sm, ctx->smem_reserved,
+                                 ctx->smem_optin, warps_per_block);
+  if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
+  WarpShape chains;
+  if (mask)
+    chains = chains_shape(compress_layout(p, false), ctx->smem_per_sm, ctx->smem_reserved,
+                          ctx->smem_optin, warps_per_block);
   // scratch: work counter, nc status words, parking slots of every warp
   const uint32_t slot_bytes =
       round16(record_bound(C / S, S, off_bytes(p->window), p->min_match) + S + 16);
-  const size_t status_end = kScratchHead + 8ull * nc;
-  const size_t park_at = (status_end + 255) & ~static_cast<size_t>(255);
+  // (then the sample's words, kSampleBytes)
+  const size_t status_end = round16_64(kScratchHead + 8ull * nc);
+  const size_t park_at = (status_end + kSampleBytes + 255) & ~static_cast<size_t>(255);
   // a launch over part of the chunks (one piece of lz_compress_host) keeps
   // the status words of the launches before it, so the scratch must not be
   // reallocated between them: it is sized for the largest grid
-  const uint64_t grid_room =
-      (c0 > 0 || c1 < nc) ? static_cast<uint64_t>(best_blocks) * ctx->sms : grid;
-  const size_t need = park_at + static_cast<size_t>(slot_bytes) * kParkSlots * wpb * grid_room;
+  const uint64_t room = (c0 > 0 || c1 < nc) ? ~0ull >> 8 : c1 - c0;
+  const uint64_t park_warps = std::max(w.warps() * w.grid(room, ctx->sms),
+                                       chains.warps() * chains.grid(room, ctx->sms));
+  const size_t need = park_at + static_cast<size_t>(slot_bytes) * kParkSlots * park_warps;
   lz_status s = reserve_scratch(ctx, need);
   if (s != LZ_OK) return s;
-  cudaError_t e = cudaMemsetAsync(ctx->scratch, 0, clear_status ? status_end : kScratchHead, st);
-  if (e != cudaSuccess) return LZ_ERR_CUDA;
+  const size_t clear_bytes = clear_status ? status_end : kScratchHead;
 
   glz::CompressArgs A{};
   A.buf.in = static_cast<const uint8_t *>(d_in);
@@ -487,7 +574,7 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
   A.buf.version = version;
   A.buf.gbase = 0;
   A.total_chunks = nc;
-  A.sm = sm;
+  A.sm = w.sm;
   A.park = static_cast<uint8_t *>(ctx->scratch) + park_at;
   A.park_slots = kParkSlots;
   A.park_slot_bytes = slot_bytes;
@@ -502,17 +589,15 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
   while (32 * nj < p->window) nj *= 2;
   // (a caller's launch shape, the pieces of lz_compress_host and the trials of
   // the autotuner keep one warp per chunk)
-  if (block_per_chunk && !warps_per_block && c0 == 0 && c1 == nc &&
-      glz::mask_parse_takes(S, p->window, p->min_match, A.buf.match) &&
-      coop_takes(ctx, nc, wpb * best_blocks * ctx->sms, S, C, std::max(nj, 4u), &A.coop))
-    return cuda_status(launch_coop(A, S, std::max(nj, 4u), static_cast<unsigned>(nc), st));
-  const unsigned g = static_cast<unsigned>(grid);
-  switch (S) {
-    case 1: e = glz::launch_compress_s1(A, nj, block, g, st); break;
-    case 2: e = glz::launch_compress_s2(A, nj, block, g, st); break;
-    default: e = glz::launch_compress_s4(A, nj, block, g, st); break;
-  }
-  return cuda_status(e);
+  const bool coop = mask && block_per_chunk && !warps_per_block && c0 == 0 && c1 == nc &&
+                    coop_takes(ctx, nc, S, C, std::max(nj, 4u), &A.coop);
+  if (mask && !coop && chains.blocks_per_sm)  // the data decide
+    A.votes = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(ctx->scratch) + status_end);
+  cudaError_t e = A.votes ? launch_sample(A, S, nj, ctx->scratch, clear_bytes, st)
+                          : cudaMemsetAsync(ctx->scratch, 0, clear_bytes, st);
+  if (e != cudaSuccess) return cuda_status(e);
+  if (coop) return cuda_status(launch_coop(A, S, std::max(nj, 4u), static_cast<unsigned>(nc), st));
+  return cuda_status(launch_parses(A, nj, mask, w, chains, c1 - c0, ctx->sms, st));
 }
 
 // Piece sizes for lz_compress_host: whole multiples of `sb` except the last
@@ -849,7 +934,8 @@ namespace {
 
 constexpr uint32_t kNoAllocMaxChunks = 65536;  // chunks per call, at most
 constexpr size_t kNoAllocHead = 16;            // [0,4) counter, [4,8) error word
-constexpr size_t kNoAllocBytes = kNoAllocHead + 8ull * kNoAllocMaxChunks;  // 512 KiB + 16
+constexpr size_t kNoAllocStatus = kNoAllocHead + 8ull * kNoAllocMaxChunks;
+constexpr size_t kNoAllocBytes = kNoAllocStatus + kSampleBytes;  // 512 KiB + 272
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -924,19 +1010,14 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
     return cuda_status(glz::launch_header(static_cast<uint8_t *>(d_out), 1u, S, offB,
                                           p->min_match, p->max_match, C, p->window,
                                           out_bytes, st));
-  const glz::CompressSmem sm = compress_layout(p, glz::kMatchExact);
-  if (static_cast<int64_t>(sm.per_warp) > nd->smem_optin) return LZ_ERR_INVALID_ARG;
-  int block = 32;
-  int64_t best_blocks = 1;
-  if (!block_shape(sm.per_warp, nd->smem_per_sm, nd->smem_reserved, nd->smem_optin, 0, &block,
-                   &best_blocks))
-    return LZ_ERR_INVALID_ARG;
-  uint64_t grid = div_up(nc, block / 32);
-  if (grid > static_cast<uint64_t>(best_blocks) * nd->sms) grid = best_blocks * nd->sms;
-  // the counter, the error word and the status words start at zero (one
-  // clear, so that an error left by an earlier failed call cannot leak in)
-  if (cudaMemsetAsync(nd->scratch, 0, kNoAllocHead + 8ull * nc, st) != cudaSuccess)
-    return LZ_ERR_CUDA;
+  const bool mask = glz::mask_parse_takes(S, p->window, p->min_match, glz::kMatchExact);
+  const WarpShape w = warp_shape(compress_layout(p, mask), nd->smem_per_sm, nd->smem_reserved,
+                                 nd->smem_optin, 0);
+  if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
+  WarpShape chains;
+  if (mask)
+    chains = warp_shape(compress_layout(p, false), nd->smem_per_sm, nd->smem_reserved,
+                        nd->smem_optin, 0);
   glz::CompressArgs A{};
   A.buf.in = static_cast<const uint8_t *>(d_in);
   A.buf.n = n_bytes;
@@ -954,24 +1035,24 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
   A.buf.in_aligned = (reinterpret_cast<uintptr_t>(d_in) % 16) == 0;
   A.buf.gbase = 0;
   A.total_chunks = nc;
-  A.sm = sm;
+  A.sm = w.sm;
   A.park = nullptr;  // no parking slots: blocking look-back
   A.park_slots = 0;
   A.park_slot_bytes = 0;
   A.ticket = reinterpret_cast<uint32_t *>(nd->scratch);
+  if (chains.blocks_per_sm) A.votes = reinterpret_cast<uint32_t *>(nd->scratch + kNoAllocStatus);
   A.err = reinterpret_cast<uint32_t *>(nd->scratch + 4);
   A.spin_limit = glz::kSpinLimit;
   A.end_chunk = static_cast<uint32_t>(nc);
   A.status = reinterpret_cast<unsigned long long *>(nd->scratch + kNoAllocHead);
   uint32_t nj = 1;
   while (32 * nj < p->window) nj *= 2;
-  cudaError_t e;
-  const unsigned g = static_cast<unsigned>(grid);
-  switch (S) {
-    case 1: e = glz::launch_compress_s1(A, nj, block, g, st); break;
-    case 2: e = glz::launch_compress_s2(A, nj, block, g, st); break;
-    default: e = glz::launch_compress_s4(A, nj, block, g, st); break;
-  }
+  // the counter, the error word and the status words start at zero (one
+  // clear, so that an error left by an earlier failed call cannot leak in)
+  const uint64_t clear_bytes = round16_64(kNoAllocHead + 8ull * nc);
+  cudaError_t e = A.votes ? launch_sample(A, S, nj, nd->scratch, clear_bytes, st)
+                          : cudaMemsetAsync(nd->scratch, 0, clear_bytes, st);
+  if (e == cudaSuccess) e = launch_parses(A, nj, mask, w, chains, nc, nd->sms, st);
   if (e != cudaSuccess) return cuda_status(e);
   noalloc_report<<<1, 32, 0, st>>>(A.err, out_bytes);
   return cuda_status(cudaGetLastError());
@@ -997,8 +1078,8 @@ struct DevBuf {
 struct BatchClass {
   uint32_t S = 1, nj = 4;
   bool mask = false, coop = false;
-  int block = 32;
-  unsigned grid = 1;
+  WarpShape shape, chains;  // one warp per chunk (see launch_parses)
+  uint64_t chunks = 0;
   glz::CompressArgs args{};
 };
 
@@ -1068,10 +1149,10 @@ lz_status batch_upload(lz_batch *b, int slot, const std::vector<T> &v, const T *
 
 // Per-warp slice covering every parameter set of a batch: each region at its
 // largest size.
-glz::CompressSmem compress_layout_max(const std::vector<lz_params> &ps, uint32_t match) {
+glz::CompressSmem compress_layout_max(const std::vector<lz_params> &ps, bool masks) {
   uint64_t in = 16, links = 16, flags = 16, pay = 16, maybe = 16;
   for (const lz_params &p : ps) {
-    const glz::CompressSmem one = compress_layout(&p, match);
+    const glz::CompressSmem one = compress_layout(&p, masks);
     in = std::max<uint64_t>(in, one.prev_off - one.in_off);
     links = std::max<uint64_t>(links, one.flags_off - one.prev_off);
     flags = std::max<uint64_t>(flags, one.pay_off - one.flags_off);
@@ -1184,15 +1265,14 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
   size_t clear = 0, park = 0;
   std::vector<size_t> clear_at, park_at;
   for (Group &g : groups) {
-    const glz::CompressSmem sm = compress_layout_max(g.ps, match);
-    if (static_cast<int64_t>(sm.per_warp) > ctx->smem_optin) return LZ_ERR_INVALID_ARG;
-    int64_t best_blocks = 1;
-    if (!block_shape(sm.per_warp, ctx->smem_per_sm, ctx->smem_reserved, ctx->smem_optin,
-                     b->warps_per_block, &g.cls.block, &best_blocks))
-      return LZ_ERR_INVALID_ARG;
-    const uint64_t wpb = g.cls.block / 32;
-    uint64_t grid = div_up(g.chunks, wpb);
-    if (grid > static_cast<uint64_t>(best_blocks) * ctx->sms) grid = best_blocks * ctx->sms;
+    WarpShape &w = g.cls.shape, &chains = g.cls.chains;
+    w = warp_shape(compress_layout_max(g.ps, g.cls.mask), ctx->smem_per_sm, ctx->smem_reserved,
+                   ctx->smem_optin, b->warps_per_block);
+    if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
+    if (g.cls.mask)
+      chains = chains_shape(compress_layout_max(g.ps, false), ctx->smem_per_sm, ctx->smem_reserved,
+                            ctx->smem_optin, b->warps_per_block);
+    g.cls.chunks = g.chunks;
     uint64_t rb_max = 0;  // a parking slot holds any item's largest record
     for (const lz_params &q : g.ps)
       rb_max = std::max<uint64_t>(rb_max, record_bound(q.chunk_bytes / q.symbol_bytes,
@@ -1202,23 +1282,25 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
     glz::CompressArgs &A = g.cls.args;
     A.n_items = static_cast<uint32_t>(g.descs.size());
     A.total_chunks = g.chunks;
-    A.sm = sm;
+    A.sm = w.sm;
     A.park_slots = kParkSlots;
     A.park_slot_bytes = round16(rb_max + 16);
     A.spin_limit = glz::kSpinLimit;
-    g.cls.grid = static_cast<unsigned>(grid);
     uint32_t c_max = 0;
     for (const lz_params &q : g.ps) c_max = std::max(c_max, q.chunk_bytes);
     if (g.cls.mask && !b->warps_per_block &&
-        coop_takes(ctx, g.chunks, wpb * best_blocks * ctx->sms, g.cls.S, c_max, g.cls.nj, &A.coop)) {
+        coop_takes(ctx, g.chunks, g.cls.S, c_max, g.cls.nj, &A.coop)) {
       g.cls.coop = true;
-      g.cls.grid = static_cast<unsigned>(g.chunks);
     }
     clear_at.push_back(clear);
-    clear += kScratchHead + 8ull * g.chunks;
+    clear += round16_64(kScratchHead + 8ull * g.chunks) + kSampleBytes;
     clear = (clear + 255) & ~static_cast<size_t>(255);
     park_at.push_back(park);
-    park += static_cast<size_t>(A.park_slot_bytes) * kParkSlots * wpb * grid;
+    // (a block per chunk parks nothing)
+    if (!g.cls.coop)
+      park += static_cast<size_t>(A.park_slot_bytes) * kParkSlots *
+              std::max(w.warps() * w.grid(g.chunks, ctx->sms),
+                       chains.warps() * chains.grid(g.chunks, ctx->sms));
     park = (park + 255) & ~static_cast<size_t>(255);
   }
   lz_status s = batch_alloc(b, kBufScratch, clear + park, &b->scratch);
@@ -1254,6 +1336,9 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
     d_items += groups[i].descs.size();
     d_base += groups[i].descs.size();
     A.ticket = reinterpret_cast<uint32_t *>(base + clear_at[i]);
+    if (groups[i].cls.mask && !groups[i].cls.coop && groups[i].cls.chains.blocks_per_sm)
+      A.votes = reinterpret_cast<uint32_t *>(base + clear_at[i] +
+                                             round16_64(kScratchHead + 8ull * A.total_chunks));
     A.status = reinterpret_cast<unsigned long long *>(base + clear_at[i] + kScratchHead);
     A.park = base + clear + park_at[i];
     b->classes.push_back(groups[i].cls);
@@ -1262,6 +1347,19 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
   b->n_empty = static_cast<uint32_t>(empties.size());
   b->clear_bytes = clear;
   return LZ_OK;
+}
+
+// One warp per chunk over the chunks of a class, as launch_parses.
+cudaError_t launch_class(BatchClass &c, int sms, cudaStream_t st) {
+  glz::CompressArgs &A = c.args;
+  auto go = [&](bool by_masks, const WarpShape &x) {
+    A.sm = x.sm;
+    return glz::launch_batch_class(A, c.S, c.nj, by_masks, x.block,
+                                   static_cast<unsigned>(x.grid(c.chunks, sms)), st);
+  };
+  cudaError_t e = A.votes ? go(false, c.chains) : cudaSuccess;
+  if (e == cudaSuccess) e = go(c.mask, c.shape);
+  return e;
 }
 
 // Class i > 0 goes to side stream (i - 1) % kBatchSides: each is ordered
@@ -1276,12 +1374,19 @@ lz_status batch_run_compress(lz_ctx *ctx, lz_batch *b, cudaStream_t st) {
   if (sides && e == cudaSuccess) e = cudaEventRecord(b->fork, st);
   for (size_t i = 0; i < sides && e == cudaSuccess; ++i)
     e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
+  auto stream_of = [&](size_t i) { return i == 0 ? st : b->side[(i - 1) % kBatchSides]; };
+  // (the samples of all classes first: behind the first class's warps they
+  // would wait for them)
+  for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+    BatchClass &c = b->classes[i];
+    if (c.args.votes) e = launch_sample(c.args, c.S, c.nj, nullptr, 0, stream_of(i));
+  }
   for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
     BatchClass &c = b->classes[i];
     c.args.err = ctx->d_err;
-    const cudaStream_t on = i == 0 ? st : b->side[(i - 1) % kBatchSides];
-    e = c.coop ? launch_coop(c.args, c.S, c.nj, c.grid, on)
-               : glz::launch_batch_class(c.args, c.S, c.nj, c.mask, c.block, c.grid, on);
+    const cudaStream_t on = stream_of(i);
+    e = c.coop ? launch_coop(c.args, c.S, c.nj, static_cast<unsigned>(c.chunks), on)
+               : launch_class(c, ctx->sms, on);
   }
   // joined also after a failed launch: the side streams must not run on
   // unordered, nor a capture be left forked
@@ -1586,7 +1691,11 @@ lz_status lz_autotune_ex(lz_ctx *ctx, const void *d_sample, uint64_t sample_byte
     for (lz_tune_trial &t : shape) {
       if (s != LZ_OK) break;
       if (t.warps_per_block &&
-          static_cast<int64_t>(compress_layout(&best, glz::kMatchExact).per_warp) * t.warps_per_block >
+          static_cast<int64_t>(
+              compress_layout(&best, glz::mask_parse_takes(best.symbol_bytes, best.window,
+                                                           best.min_match, glz::kMatchExact))
+                  .per_warp) *
+                  t.warps_per_block >
               ctx->smem_optin)
         continue;  // this shape does not fit a block
       run(t);
