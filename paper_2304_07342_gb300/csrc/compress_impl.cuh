@@ -1247,7 +1247,7 @@ __device__ __forceinline__ uint32_t find_item(const CompressArgs &A, uint64_t g,
 template <int S, int NJ, bool MASK>
 __global__ void __maxnreg__(reg_limit(S, NJ, MASK)) compress_batch_kernel(const CompressArgs A) {
   extern __shared__ __align__(128) uint8_t smem[];
-  __shared__ BufDesc descs[8];
+  __shared__ BufDesc descs[kBatchDescBytes / sizeof(BufDesc)];
   if (!chosen<S, NJ, MASK>(A)) return;
   const uint32_t lane = threadIdx.x & 31;
   BufDesc &B = descs[threadIdx.x >> 5];

@@ -133,6 +133,10 @@ struct BufDesc {
   uint64_t gbase;       // index of this buffer's chunk 0 among all chunks
 };
 
+// Shared memory of a batch's block beside its warps' slices: a descriptor for
+// each of up to eight warps.
+constexpr uint32_t kBatchDescBytes = 8 * sizeof(BufDesc);
+
 struct CompressArgs {
   BufDesc buf;                 // single-buffer launch
   const BufDesc *items;        // batched launch (nullptr for a single buffer)

@@ -218,13 +218,14 @@ glz::CompressSmem compress_layout(const lz_params *p, bool masks) {
 // slice of `per_warp` bytes: `want` warps per block (1, 2, 4 or 8) when
 // given, else the choice among 1, 2, 4 that keeps the most warps resident
 // under the per-SM shared-memory limit (each block also reserves some).
-// False when not even one block fits.
-bool block_shape(int64_t per_warp, int smem_per_sm, int smem_reserved, int smem_optin,
-                 uint32_t want, int *block, int64_t *blocks_per_sm) {
+// `fixed`: the kernel's own shared memory per block.  False when not even one
+// block fits.
+bool block_shape(int64_t per_warp, int64_t fixed, int smem_per_sm, int smem_reserved,
+                 int smem_optin, uint32_t want, int *block, int64_t *blocks_per_sm) {
   int64_t best_warps = 0;
   for (int wpb = 1; wpb <= 8; wpb *= 2) {
     if (want ? static_cast<uint32_t>(wpb) != want : wpb > kCompressWarps) continue;
-    const int64_t per_block = per_warp * wpb + smem_reserved;
+    const int64_t per_block = per_warp * wpb + fixed + smem_reserved;
     if (per_block - smem_reserved > smem_optin) break;
     int64_t blocks = smem_per_sm / per_block;
     if (blocks > 32) blocks = 32;
@@ -251,12 +252,12 @@ struct WarpShape {
   }
 };
 
-WarpShape warp_shape(const glz::CompressSmem &sm, int smem_per_sm, int smem_reserved,
-                     int smem_optin, uint32_t want) {
+WarpShape warp_shape(const glz::CompressSmem &sm, int64_t fixed, int smem_per_sm,
+                     int smem_reserved, int smem_optin, uint32_t want) {
   WarpShape w;
   w.sm = sm;
   if (static_cast<int64_t>(sm.per_warp) > smem_optin ||
-      !block_shape(sm.per_warp, smem_per_sm, smem_reserved, smem_optin, want, &w.block,
+      !block_shape(sm.per_warp, fixed, smem_per_sm, smem_reserved, smem_optin, want, &w.block,
                    &w.blocks_per_sm))
     w.blocks_per_sm = 0;
   return w;
@@ -264,10 +265,10 @@ WarpShape warp_shape(const glz::CompressSmem &sm, int smem_per_sm, int smem_rese
 
 // The chains beside a parse by masks, of whose launch shape `want` is: their
 // slice is larger, so they may need the library's own choice.
-WarpShape chains_shape(const glz::CompressSmem &sm, int smem_per_sm, int smem_reserved,
-                       int smem_optin, uint32_t want) {
-  WarpShape w = warp_shape(sm, smem_per_sm, smem_reserved, smem_optin, want);
-  if (!w.blocks_per_sm) w = warp_shape(sm, smem_per_sm, smem_reserved, smem_optin, 0);
+WarpShape chains_shape(const glz::CompressSmem &sm, int64_t fixed, int smem_per_sm,
+                       int smem_reserved, int smem_optin, uint32_t want) {
+  WarpShape w = warp_shape(sm, fixed, smem_per_sm, smem_reserved, smem_optin, want);
+  if (!w.blocks_per_sm) w = warp_shape(sm, fixed, smem_per_sm, smem_reserved, smem_optin, 0);
   return w;
 }
 
@@ -531,12 +532,12 @@ lz_status compress_locked(lz_ctx *ctx, const void *d_in, uint64_t n_bytes, const
                                           p->window, out_bytes, st));
 
   const bool mask = glz::mask_parse_takes(S, p->window, p->min_match, kernel_match(match));
-  const WarpShape w = warp_shape(compress_layout(p, mask), ctx->smem_per_sm, ctx->smem_reserved,
+  const WarpShape w = warp_shape(compress_layout(p, mask), 0, ctx->smem_per_sm, ctx->smem_reserved,
                                  ctx->smem_optin, warps_per_block);
   if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
   WarpShape chains;
   if (mask)
-    chains = chains_shape(compress_layout(p, false), ctx->smem_per_sm, ctx->smem_reserved,
+    chains = chains_shape(compress_layout(p, false), 0, ctx->smem_per_sm, ctx->smem_reserved,
                           ctx->smem_optin, warps_per_block);
   // scratch: work counter, nc status words, parking slots of every warp
   const uint32_t slot_bytes =
@@ -1011,12 +1012,12 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
                                           p->min_match, p->max_match, C, p->window,
                                           out_bytes, st));
   const bool mask = glz::mask_parse_takes(S, p->window, p->min_match, glz::kMatchExact);
-  const WarpShape w = warp_shape(compress_layout(p, mask), nd->smem_per_sm, nd->smem_reserved,
+  const WarpShape w = warp_shape(compress_layout(p, mask), 0, nd->smem_per_sm, nd->smem_reserved,
                                  nd->smem_optin, 0);
   if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
   WarpShape chains;
   if (mask)
-    chains = warp_shape(compress_layout(p, false), nd->smem_per_sm, nd->smem_reserved,
+    chains = warp_shape(compress_layout(p, false), 0, nd->smem_per_sm, nd->smem_reserved,
                         nd->smem_optin, 0);
   glz::CompressArgs A{};
   A.buf.in = static_cast<const uint8_t *>(d_in);
@@ -1266,12 +1267,18 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
   std::vector<size_t> clear_at, park_at;
   for (Group &g : groups) {
     WarpShape &w = g.cls.shape, &chains = g.cls.chains;
-    w = warp_shape(compress_layout_max(g.ps, g.cls.mask), ctx->smem_per_sm, ctx->smem_reserved,
-                   ctx->smem_optin, b->warps_per_block);
+    w = warp_shape(compress_layout_max(g.ps, g.cls.mask), glz::kBatchDescBytes, ctx->smem_per_sm,
+                   ctx->smem_reserved, ctx->smem_optin, b->warps_per_block);
+    // (a stated shape that only the descriptors keep from fitting gives way)
+    if (!w.blocks_per_sm && warp_shape(w.sm, 0, ctx->smem_per_sm, ctx->smem_reserved,
+                                       ctx->smem_optin, b->warps_per_block).blocks_per_sm)
+      w = warp_shape(w.sm, glz::kBatchDescBytes, ctx->smem_per_sm, ctx->smem_reserved,
+                     ctx->smem_optin, 0);
     if (!w.blocks_per_sm) return LZ_ERR_INVALID_ARG;
     if (g.cls.mask)
-      chains = chains_shape(compress_layout_max(g.ps, false), ctx->smem_per_sm, ctx->smem_reserved,
-                            ctx->smem_optin, b->warps_per_block);
+      chains = chains_shape(compress_layout_max(g.ps, false), glz::kBatchDescBytes,
+                            ctx->smem_per_sm, ctx->smem_reserved, ctx->smem_optin,
+                            b->warps_per_block);
     g.cls.chunks = g.chunks;
     uint64_t rb_max = 0;  // a parking slot holds any item's largest record
     for (const lz_params &q : g.ps)
