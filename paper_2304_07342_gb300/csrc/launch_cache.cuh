@@ -11,14 +11,21 @@ namespace glz {
 
 // Launch-shape cache for one kernel instance, one entry per device: the
 // shared-memory opt-in (cudaFuncSetAttribute acts on the current device's
-// context only) and the occupancy query are redone whenever the block or
-// shared-memory size changes on that device.
+// context only), which is only ever raised -- another thread may be about to
+// launch the instance with the larger size -- and the resident blocks of the
+// last few shapes.
 constexpr int kMaxDevices = 64;
+constexpr int kShapes = 4;
 
 struct LaunchCache {
-  struct Entry {
-    int block = -1, per_sm = 0, sms = 0;
+  struct Shape {
+    int block = -1, per_sm = 0;
     size_t smem = 0;
+  };
+  struct Entry {
+    int sms = 0, next = 0;
+    size_t granted = 0;
+    Shape shapes[kShapes];
   };
   std::mutex mu;
   Entry dev[kMaxDevices];
@@ -35,21 +42,27 @@ static cudaError_t resident_blocks(LaunchCache &lc, K kern, int block,
   if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(lc.mu);
   LaunchCache::Entry &c = lc.dev[dev];
-  if (c.block == block && c.smem == smem) {
-    *per_sm = c.per_sm;
-    *sms = c.sms;
-    return cudaSuccess;
+  for (const LaunchCache::Shape &s : c.shapes)
+    if (s.block == block && s.smem == smem) {
+      *per_sm = s.per_sm;
+      *sms = c.sms;
+      return cudaSuccess;
+    }
+  if (smem > c.granted) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    c.granted = smem;
   }
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, block, smem);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  c.block = block;
-  c.smem = smem;
-  c.per_sm = *per_sm;
+  LaunchCache::Shape &s = c.shapes[c.next];
+  c.next = (c.next + 1) % kShapes;
+  s.block = block;
+  s.smem = smem;
+  s.per_sm = *per_sm;
   c.sms = *sms;
   return cudaSuccess;
 }
