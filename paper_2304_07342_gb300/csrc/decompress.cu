@@ -195,7 +195,8 @@ __device__ __forceinline__ void copy_s2g(uint8_t *dst, const uint8_t *src,
 struct Slice {
   uint64_t *bar;
   uint8_t *marks;           // per position: 0 inside a token, 1 literal start, 2 pointer start
-  uint16_t *dist;           // per position of a round: how far back its source lies
+  uint16_t *dist;           // per position of a round: how far back its source lies (over fl,
+                            // which only the first phase reads)
   uint8_t *hi;              // high bytes of (offset - 1), or nullptr
   uint8_t *fl;              // a copy of the record's flag bytes
   uint8_t *io;              // output image + staged record, or nullptr (decode

@@ -199,8 +199,8 @@ struct DecItem {
 // Per-warp shared-memory slice of the decoder (byte offsets, 16-byte
 // aligned): an mbarrier, one mark byte per position of the chunk (0 inside
 // a token, 1 where a literal starts, 2 where a pointer starts), a copy of
-// the record's flag bytes, a round's source distances, the high bytes of (offset - 1) when one-byte
-// symbols carry two-byte offsets, then -- when they fit -- the io area:
+// the record's flag bytes, later a round's source distances, the high bytes of
+// (offset - 1) when one-byte symbols carry two-byte offsets, then -- when they fit -- the io area:
 // the chunk's output image from its start, with the record staged at its
 // end.  When no pointer takes more payload bytes than the symbols it
 // covers (S * m >= 1 + offB for every stream; `shared`), the output
@@ -213,7 +213,7 @@ struct DecodeLayout {
   uint32_t mark_bytes;
   uint32_t flags_off;  // flag bytes of one record (+ 16 slack)
   uint32_t flag_bytes;
-  uint32_t dist_off;   // 128 source distances (u16), one round of positions, and a zero
+  uint32_t dist_off;   // kDistBytes over the flag bytes (second phase)
   uint32_t hi_off;     // k bytes (one-byte symbols, two-byte offsets) or none
   uint32_t io_off;     // output image + staged record
   uint32_t io_bytes;
@@ -228,6 +228,9 @@ __host__ __device__ inline uint64_t decode_record_bound(uint64_t k, uint32_t S, 
   const uint64_t extra = (1u + offB > S * m) ? (1u + offB - S * m) : 0u;
   return (k + 7) / 8 + static_cast<uint64_t>(S) * k + extra * (k / m) + (S - 1);
 }
+
+// A round's source distances (128 u16) and a zero after them.
+constexpr uint32_t kDistBytes = 256 + 16;
 
 // Slack of the io area past the staged record (its end is at most this
 // many bytes before the area's end, minus 15 for alignment).
@@ -245,10 +248,12 @@ __host__ __device__ inline DecodeLayout decode_layout(uint64_t kmax, uint64_t cm
   L.mark_bytes = static_cast<uint32_t>((kmax + 127) & ~127ull);
   at += L.mark_bytes;
   L.flags_off = static_cast<uint32_t>(at);
+  // (the second phase reads no flags: its distances take their place, which
+  // keeps 21 warps resident on streams of 8 KiB chunks, 20 beside them)
   L.flag_bytes = static_cast<uint32_t>(((kmax + 7) / 8 + 15) & ~15ull) + 16;
+  if (L.flag_bytes < kDistBytes) L.flag_bytes = kDistBytes;
+  L.dist_off = L.flags_off;
   at += L.flag_bytes;
-  L.dist_off = static_cast<uint32_t>(at);
-  at += 256 + 16;
   L.hi_off = static_cast<uint32_t>(at);
   if (hi) at += (kmax + 15) & ~15ull;
   const uint64_t base = at;
