@@ -1101,6 +1101,7 @@ struct lz_batch {
   // launches of the classes after the first, forked from and joined to the
   // caller's stream
   cudaStream_t side[kBatchSides] = {};
+  int side_priority = 0;
   cudaEvent_t fork = nullptr, join[kBatchSides] = {};
   std::mutex run_mu;  // a run's fork and join use the batch's events
   void *scratch = nullptr;
@@ -1188,6 +1189,39 @@ void batch_streams_free(lz_batch *b) {
     if (b->side[i]) cudaStreamDestroy(b->side[i]);
   }
   if (b->fork) cudaEventDestroy(b->fork);
+}
+
+// The side streams and events that the batch's classes need, the streams with
+// the priority of `st`: a run's launches all have that of the caller's stream.
+// (Creating a stream is no work on one, so it is not kept out of a capture.)
+cudaError_t batch_sides(lz_batch *b, size_t classes, cudaStream_t st) {
+  const int sides = static_cast<int>(std::min<size_t>(classes > 1 ? classes - 1 : 0, kBatchSides));
+  if (sides == 0) return cudaSuccess;
+  int priority = 0;
+  cudaError_t e = cudaStreamGetPriority(st, &priority);
+  if (e != cudaSuccess) return e;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  if ((e = cudaThreadExchangeStreamCaptureMode(&mode)) != cudaSuccess) return e;
+  if (!b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  for (int i = 0; i < sides && e == cudaSuccess; ++i) {
+    if (b->side[i] && b->side_priority != priority) {
+      cudaStreamDestroy(b->side[i]);  // (what runs there still ends)
+      b->side[i] = nullptr;
+    }
+    if (!b->side[i])
+      e = cudaStreamCreateWithPriority(&b->side[i], cudaStreamNonBlocking, priority);
+    if (e == cudaSuccess && !b->join[i])
+      e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
+  }
+  if (b->side_priority != priority)  // those that this run does not need
+    for (int i = sides; i < kBatchSides; ++i)
+      if (b->side[i]) {
+        cudaStreamDestroy(b->side[i]);
+        b->side[i] = nullptr;
+      }
+  b->side_priority = priority;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  return e;
 }
 
 // A compression batch is one launch per class of buffers (BatchClass), the
@@ -1324,15 +1358,7 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
   if ((s = batch_upload(b, kBufItems, descs, &d_items)) != LZ_OK) return s;
   if ((s = batch_upload(b, kBufBases, bases, &d_base)) != LZ_OK) return s;
   if ((s = batch_upload(b, kBufEmpties, empties, &d_empty)) != LZ_OK) return s;
-  cudaError_t e = cudaSuccess;
-  const int sides = static_cast<int>(std::min<size_t>(groups.empty() ? 0 : groups.size() - 1,
-                                                      kBatchSides));
-  if (sides && !b->fork) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-  for (int i = 0; i < sides && e == cudaSuccess; ++i) {
-    if (!b->side[i]) e = cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking);
-    if (e == cudaSuccess && !b->join[i])
-      e = cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming);
-  }
+  const cudaError_t e = batch_sides(b, groups.size(), b->stream);
   if (e != cudaSuccess) return cuda_status(e);
   b->classes.clear();
   uint8_t *base = static_cast<uint8_t *>(b->scratch);
@@ -1377,8 +1403,10 @@ lz_status batch_run_compress(lz_ctx *ctx, lz_batch *b, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (b->n_empty) e = glz::launch_batch_empties(b->d_empty, b->n_empty, st);
   const size_t n = b->classes.size();
+  if (e == cudaSuccess) e = batch_sides(b, n, st);
+  if (e != cudaSuccess) return cuda_status(e);
   const size_t sides = n > 1 ? std::min<size_t>(n - 1, kBatchSides) : 0;
-  if (sides && e == cudaSuccess) e = cudaEventRecord(b->fork, st);
+  if (sides) e = cudaEventRecord(b->fork, st);
   for (size_t i = 0; i < sides && e == cudaSuccess; ++i)
     e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
   auto stream_of = [&](size_t i) { return i == 0 ? st : b->side[(i - 1) % kBatchSides]; };
