@@ -220,7 +220,7 @@ lz_status lz_decompress(lz_ctx *ctx, const void *d_in, uint64_t in_bytes,
 /* Compression for callers that cannot allocate device memory (no paper
  * counterpart; an addition of this library).  Same stream as lz_compress,
  * on the current device, with no context: the scratch is a fixed device
- * array inside the library (512 KiB + 16 B, held by every GPU that loads
+ * array inside the library (512 KiB + 272 B, held by every GPU that loads
  * the library until the process exits), so the call allocates nothing and
  * n_bytes may span at most 65536 chunks (LZ_ERR_INVALID_ARG beyond that).
  * The caller passes inputs and outputs as for lz_compress.  Device-side
@@ -232,10 +232,11 @@ lz_status lz_decompress(lz_ctx *ctx, const void *d_in, uint64_t in_bytes,
  * on one stream are fine.  The first call on a device looks up the array's
  * device address (and launch limits); make that first call before any
  * stream capture.  Under CUDA's lazy module loading (the default) the first
- * launch of each kernel variant loads its code onto the device, which takes
+ * use of each kernel variant loads its code onto the device, which takes
  * device memory: before entering a region where nothing may be allocated,
  * make one call for every symbol size and window class it will use (window
- * classes: W <= 32, <= 64, <= 128, <= 256, <= 512, <= 1024), plus one with
+ * classes: W <= 32, <= 64, <= 128, <= 256, <= 512, <= 1024), which loads all
+ * variants of that class, plus one with
  * n_bytes = 0 if empty inputs occur.  Slower than lz_compress on inputs with
  * uneven chunks: a chunk whose offset is not yet known waits instead of
  * moving on. */

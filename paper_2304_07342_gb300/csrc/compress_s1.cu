@@ -13,4 +13,5 @@ cudaError_t launch_sample_s1(const CompressArgs &A, uint32_t nj, void *clear, ui
                              cudaStream_t stream) {
   return launch_sample_t<1>(A, nj, clear, clear_bytes, stream);
 }
+cudaError_t load_parses_s1(uint32_t nj) { return load_parses_t<1>(nj); }
 }  // namespace glz

@@ -6,6 +6,7 @@
 #include <cstdint>
 #include <cstring>
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -20,6 +21,9 @@ cudaError_t launch_compress_s2(const CompressArgs &A, uint32_t nj, bool mask, in
                                unsigned grid, cudaStream_t stream);
 cudaError_t launch_compress_s4(const CompressArgs &A, uint32_t nj, bool mask, int block,
                                unsigned grid, cudaStream_t stream);
+cudaError_t load_parses_s1(uint32_t nj);
+cudaError_t load_parses_s2(uint32_t nj);
+cudaError_t load_parses_s4(uint32_t nj);
 cudaError_t launch_sample_s1(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
                              cudaStream_t stream);
 cudaError_t launch_sample_s2(const CompressArgs &A, uint32_t nj, void *clear, uint64_t clear_bytes,
@@ -954,6 +958,7 @@ struct NoAllocDevice {
   bool ready = false;
   unsigned char *scratch = nullptr;  // device address of g_noalloc_scratch
   int smem_optin = 0, smem_per_sm = 0, smem_reserved = 0, sms = 0;
+  std::atomic<uint32_t> loaded{0};  // symbol sizes x window classes whose kernels are loaded
 };
 
 // Per-device set-up, done once with that device current: the device address
@@ -1048,6 +1053,18 @@ extern "C" lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes,
   A.status = reinterpret_cast<unsigned long long *>(nd->scratch + kNoAllocHead);
   uint32_t nj = 1;
   while (32 * nj < p->window) nj *= 2;
+  // the first call of a symbol size and window class loads every kernel of it,
+  // also those that another min_match or other data take
+  uint32_t cls = 0;
+  while ((1u << cls) < nj) ++cls;
+  const uint32_t bit = 1u << (8 * (S / 2) + cls);
+  if (!(nd->loaded.load() & bit)) {
+    const cudaError_t l = S == 1   ? glz::load_parses_s1(nj)
+                          : S == 2 ? glz::load_parses_s2(nj)
+                                   : glz::load_parses_s4(nj);
+    if (l != cudaSuccess) return cuda_status(l);
+    nd->loaded.fetch_or(bit);
+  }
   // the counter, the error word and the status words start at zero (one
   // clear, so that an error left by an earlier failed call cannot leak in)
   const uint64_t clear_bytes = round16_64(kNoAllocHead + 8ull * nc);

@@ -52,4 +52,30 @@ static cudaError_t launch_sample_t(const CompressArgs &A, uint32_t nj, void *cle
   return go(sample_kernel<S, 16>);
 }
 
+// Load the code of every kernel that a call with symbols of S bytes and windows
+// of 32 * nj symbols can launch (loading is lazy and takes device memory).
+template <int S, int NJ>
+static cudaError_t load_parses_nj() {
+  cudaFuncAttributes a;
+  cudaError_t e = cudaFuncGetAttributes(&a, compress_kernel<S, NJ, false>);
+  if constexpr (32 * NJ <= kMaskMaxWindow) {
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, compress_kernel<S, NJ, true>);
+    if (e == cudaSuccess)
+      e = cudaFuncGetAttributes(&a, sample_kernel<S, (NJ <= 4 ? 4 : NJ)>);
+  }
+  return e;
+}
+
+template <int S>
+static cudaError_t load_parses_t(uint32_t nj) {
+  switch (nj) {
+    case 1: return load_parses_nj<S, 1>();
+    case 2: return load_parses_nj<S, 2>();
+    case 4: return load_parses_nj<S, 4>();
+    case 8: return load_parses_nj<S, 8>();
+    case 16: return load_parses_nj<S, 16>();
+    default: return load_parses_nj<S, 32>();
+  }
+}
+
 }  // namespace glz
