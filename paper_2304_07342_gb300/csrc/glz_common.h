@@ -158,6 +158,20 @@ struct CompressArgs {
   uint32_t end_chunk;          // single buffer: chunks [first_ticket, end_chunk) are taken
 };
 
+// The classes of a batch between whose parses a sample chooses: three symbol
+// sizes, three window classes.
+struct SampleClass {
+  const BufDesc *items;
+  const uint64_t *item_base;
+  uint64_t total_chunks;
+  uint32_t *votes;
+  uint32_t n_items, S, nj;
+};
+struct SampleList {
+  SampleClass e[9];
+  uint32_t n;
+};
+
 // Placement of one shard stream inside a whole-input stream (lz_stitch).
 struct StitchArgs {
   const uint8_t *shard;   // 8-byte aligned

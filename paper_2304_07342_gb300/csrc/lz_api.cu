@@ -37,6 +37,7 @@ cudaError_t launch_coop_s4(const CompressArgs &A, uint32_t nw, unsigned grid, cu
 cudaError_t coop_blocks_s1(uint32_t nw, uint32_t smem, int *per_sm);
 cudaError_t coop_blocks_s2(uint32_t nw, uint32_t smem, int *per_sm);
 cudaError_t coop_blocks_s4(uint32_t nw, uint32_t smem, int *per_sm);
+cudaError_t launch_sample_batch(const SampleList &L, cudaStream_t stream);
 cudaError_t launch_batch_empties(const BufDesc *empties, uint32_t n, cudaStream_t stream);
 cudaError_t launch_batch_class(const CompressArgs &A, uint32_t S, uint32_t nj, bool mask,
                                int block, unsigned grid, cudaStream_t stream);
@@ -1112,6 +1113,7 @@ struct lz_batch {
   DevBuf bufs[kBufCount];         // device allocations owned by the batch
   // compression
   std::vector<BatchClass> classes;  // most work first
+  glz::SampleList samples{};        // those whose data decide
   const glz::BufDesc *d_empty = nullptr;
   uint32_t n_empty = 0;
   size_t clear_bytes = 0;
@@ -1378,6 +1380,7 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
   const cudaError_t e = batch_sides(b, groups.size(), b->stream);
   if (e != cudaSuccess) return cuda_status(e);
   b->classes.clear();
+  b->samples.n = 0;
   uint8_t *base = static_cast<uint8_t *>(b->scratch);
   for (size_t i = 0; i < groups.size(); ++i) {
     glz::CompressArgs &A = groups[i].cls.args;
@@ -1391,6 +1394,9 @@ lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_
                                              round16_64(kScratchHead + 8ull * A.total_chunks));
     A.status = reinterpret_cast<unsigned long long *>(base + clear_at[i] + kScratchHead);
     A.park = base + clear + park_at[i];
+    if (A.votes)
+      b->samples.e[b->samples.n++] = {A.items, A.item_base, A.total_chunks, A.votes, A.n_items,
+                                      groups[i].cls.S, groups[i].cls.nj};
     b->classes.push_back(groups[i].cls);
   }
   b->d_empty = d_empty;
@@ -1407,8 +1413,10 @@ cudaError_t launch_class(BatchClass &c, int sms, cudaStream_t st) {
     return glz::launch_batch_class(A, c.S, c.nj, by_masks, x.block,
                                    static_cast<unsigned>(x.grid(c.chunks, sms)), st);
   };
-  cudaError_t e = A.votes ? go(false, c.chains) : cudaSuccess;
-  if (e == cudaSuccess) e = go(c.mask, c.shape);
+  // (masks first, unlike a single buffer: what the first class takes of the GPU
+  // before the others come decides how long a small batch lasts)
+  cudaError_t e = go(c.mask, c.shape);
+  if (e == cudaSuccess && A.votes) e = go(false, c.chains);
   return e;
 }
 
@@ -1423,16 +1431,13 @@ lz_status batch_run_compress(lz_ctx *ctx, lz_batch *b, cudaStream_t st) {
   if (e == cudaSuccess) e = batch_sides(b, n, st);
   if (e != cudaSuccess) return cuda_status(e);
   const size_t sides = n > 1 ? std::min<size_t>(n - 1, kBatchSides) : 0;
-  if (sides) e = cudaEventRecord(b->fork, st);
+  // (the samples of all classes first: behind the first class's warps they
+  // would wait for them)
+  if (b->samples.n) e = glz::launch_sample_batch(b->samples, st);
+  if (sides && e == cudaSuccess) e = cudaEventRecord(b->fork, st);
   for (size_t i = 0; i < sides && e == cudaSuccess; ++i)
     e = cudaStreamWaitEvent(b->side[i], b->fork, 0);
   auto stream_of = [&](size_t i) { return i == 0 ? st : b->side[(i - 1) % kBatchSides]; };
-  // (the samples of all classes first: behind the first class's warps they
-  // would wait for them)
-  for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
-    BatchClass &c = b->classes[i];
-    if (c.args.votes) e = launch_sample(c.args, c.S, c.nj, nullptr, 0, stream_of(i));
-  }
   for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
     BatchClass &c = b->classes[i];
     c.args.err = ctx->d_err;

@@ -32,6 +32,10 @@ constexpr uint32_t kSampleBlock = 256;
 // keys.
 __host__ __device__ constexpr uint32_t sample_symbols(int nw) { return 32 * nw + 4 * kSamplePositions + 32; }
 
+// By sampling warp w: the chunk (in 2^32ths of all) and the place in it.
+__device__ __forceinline__ uint32_t sample_hash(uint32_t w) { return (2 * w + 1) * 0x9E3779B1u; }
+__device__ __forceinline__ uint32_t sample_place(uint32_t h) { return (h ^ (h >> 15)) * 0x85EBCA77u; }
+
 // The number of positions inside the window of position p (>= 32 * NW) that
 // carry its key, its first g symbols.
 template <int S, int NW>

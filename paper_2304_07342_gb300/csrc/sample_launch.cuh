@@ -18,17 +18,9 @@ __global__ void __launch_bounds__(kSampleBlock) sample_kernel(const __grid_const
     clear[i] = make_uint4(0, 0, 0, 0);
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, w = blockIdx.x * 8 + warp;
   if (w >= kSampleWarps) return;
-  // a chunk and a place in it, by a hash of the warp's number
-  const uint32_t h = (2 * w + 1) * 0x9E3779B1u, r = (h ^ (h >> 15)) * 0x85EBCA77u;
-  uint32_t v;
-  if (A.items) {
-    const uint64_t g = (A.total_chunks * h) >> 32;  // (fewer than 2^32 chunks)
-    const BufDesc B = A.items[find_item(A, g, lane)];
-    v = sample_piece<S, NW>(B, static_cast<uint32_t>(g - B.gbase), r, pieces[warp], lane);
-  } else {
-    const uint32_t first = A.first_ticket < A.end_chunk ? A.first_ticket : 0u;
-    v = sample_piece<S, NW>(A.buf, first + __umulhi(h, A.end_chunk - first), r, pieces[warp], lane);
-  }
+  const uint32_t h = sample_hash(w), first = A.first_ticket < A.end_chunk ? A.first_ticket : 0u;
+  const uint32_t v = sample_piece<S, NW>(A.buf, first + __umulhi(h, A.end_chunk - first),
+                                         sample_place(h), pieces[warp], lane);
   if (lane == 0) A.votes[w] = v;
 }
 
