@@ -25,10 +25,10 @@ beside the exact one on 256 MiB of uint16 quantization codes; `huffman` --
 the paper's use case (section 4.5), Huffman coding after LZSS, on the same
 codes; `batched` --
 10,000 uneven buffers (4 KiB-16 MiB, four
-kinds, about 20 GB) compressed and decompressed by one persistent launch
-under a CUDA graph vs one plain launch per buffer -- and `served` -- a
+kinds, about 20 GB) compressed and decompressed by batched launches
+under a CUDA graph vs one call per buffer -- and `served` -- a
 Poisson request stream (2000 requests/s for 60 s, the full trace; --served
-sets the seconds) under continuous batching vs one launch per request, with
+sets the seconds) under continuous batching vs one call per request, with
 p50/p99 latency, then a load sweep to saturation.
 
 `--impl reference` times the CPU oracle (the plain definition) on a bounded
@@ -139,7 +139,8 @@ class ClockSampler:
 # The compression kernel's sources: a DRAM traffic figure from an ncu capture
 # holds only while these are unchanged.
 KERNEL_SOURCES = ("compress_impl.cuh", "compress_launch.cuh", "compress_s4.cu",
-                  "glz_common.h", "glz_device.cuh", "mask_parse.cuh")
+                  "glz_common.h", "glz_device.cuh", "launch_cache.cuh", "mask_parse.cuh",
+                  "sample.cuh", "sample_launch.cuh")
 PROFILE = os.path.join(ROOT, "profiles", "compress_kernel_field-256MiB.md")
 
 
@@ -369,7 +370,8 @@ def run_gpu(args):
                      "algorithmic_bytes": k_bytes,
                      "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)"},
         "e2e": e2e,
-        "gpu_launches": args.steps * len(items) * 2,
+        # per buffer: the sample, the two parses it chooses from, the decoder
+        "gpu_launches": args.steps * len(items) * 4,
         "stream_version2": v2,
         "clocks": clk.summary(),
     }
@@ -624,8 +626,8 @@ def _sweep(torch, codec, args, reps: int = 3):
 
 
 def _batched(torch, codec, args, n_buffers: int = 10_000):
-    """Many uneven buffers: one persistent launch under a CUDA graph vs one
-    plain launch per buffer (compress and decompress of every buffer)."""
+    """Many uneven buffers: batched launches under a CUDA graph vs one call
+    per buffer (compress and decompress of every buffer)."""
     from paper_2304_07342_gb300 import batch
     t = time.perf_counter()
     tuning = []
@@ -643,10 +645,10 @@ def _batched(torch, codec, args, n_buffers: int = 10_000):
 
 
 def _served(torch, codec, args, seconds: float, budget: int = 40 * 10 ** 9):
-    """Poisson request stream: continuous batching vs one plain launch per
+    """Poisson request stream: continuous batching vs one call per
     request, same trace, same HBM budget.  Then a load sweep: traces of
     about 6,000 requests at rising arrival rates, each run both ways, to
-    show where one launch per request saturates."""
+    show where one call per request saturates."""
     from paper_2304_07342_gb300 import serve
     tr = serve.build_trace(torch, codec, rate=2000.0, duration=seconds, seed=args.seed)
     b = serve.run_batched(torch, codec, tr, budget_bytes=budget)

@@ -119,8 +119,12 @@ uint64_t lz_compressed_bound(uint64_t n_bytes, const lz_params *p);
 
 /* Compress n_bytes at d_in (n_bytes % S == 0; n_bytes == 0 allowed) into
  * d_out (capacity out_cap bytes) and store the stream size in *d_out_bytes
- * (a device uint64, 8-byte aligned).  One kernel launch (plus a scratch
- * clear); d_in is staged with TMA bulk copies when it is 16-byte aligned.
+ * (a device uint64, 8-byte aligned).  A scratch clear and one kernel launch;
+ * or, where the parse depends on the data (exact matchers, W <= 512, more
+ * chunks than blocks that are resident), a small launch that clears the
+ * scratch and samples the input, then two launches, one parse each, of which
+ * the one that the sample did not choose ends at once.  Both give the same
+ * stream.  d_in is staged with TMA bulk copies when it is 16-byte aligned.
  * Returns LZ_ERR_BUFFER_TOO_SMALL synchronously when out_cap cannot even
  * hold header + table + index; if the records do not fit, the stream is
  * incomplete, *d_out_bytes still receives the size that was needed and
@@ -148,9 +152,14 @@ typedef struct lz_options {
                        payload_bytes.  lz_decompress reads both.       */
   uint32_t warps_per_block; /* compression launch shape: warps per block
                        (one chunk per warp at a time): 1, 2, 4 or 8;
-                       0 = the library's choice, the one that keeps the
-                       most warps resident.  It changes how chunks are
-                       spread over the GPU, never the stream.          */
+                       0 = the library's choice: the one that keeps the
+                       most warps resident, or, when the chunks are few,
+                       a block of eight warps per chunk.  It changes how
+                       chunks are spread over the GPU, never the stream.
+                       (A shape that fits one of a launch's parses but
+                       not the other leaves the other's to the library,
+                       as does one that fits a batch only without the
+                       batch's own descriptors.)                       */
 } lz_options;
 
 /* lz_compress with options (opt may be NULL: the defaults).
@@ -248,14 +257,17 @@ lz_status lz_compress_noalloc(const void *d_in, uint64_t n_bytes, const lz_param
  * A batch is planned once on the host (lz_batch_create: validates every item,
  * uploads per-buffer descriptors, sizes and allocates its own scratch) and
  * run any number of times (lz_batch_run: decompression is one persistent
- * kernel over the chunks of all streams; compression is a scratch clear and
- * one kernel per class of buffers -- symbol size, parse, range of windows --
- * whose warps take chunks from the class's work counter, the classes side by
- * side on streams of the batch that start after what the caller's stream
- * holds and that the caller's stream waits for; no host synchronisation, no
- * allocation, so a run can be captured in a CUDA graph and replayed).  The result of every item is byte-identical to
- * lz_compress / lz_decompress of that item alone.  Device errors are sticky
- * in the context, as for the single-buffer calls. */
+ * kernel over the chunks of all streams; compression is a scratch clear, one
+ * launch that samples the data, and one or two kernels per class of buffers
+ * (symbol size, range of windows, and the parses the sample chooses from)
+ * whose warps take chunks from the class's work counter.  The classes run side
+ * by side on streams of the batch that start after what the caller's stream
+ * holds, that the caller's stream waits for, and that have its priority.  No
+ * host synchronisation, no allocation, so a run can be captured in a CUDA
+ * graph and replayed; the first run from a stream of another priority than the
+ * batch last ran at makes the batch's streams anew).  The result of every item
+ * is byte-identical to lz_compress / lz_decompress of that item alone.  Device
+ * errors are sticky in the context, as for the single-buffer calls. */
 typedef struct lz_batch_item {
   const void *d_in;      /* input (compress) or stream (decompress)         */
   uint64_t in_bytes;
@@ -320,9 +332,10 @@ void lz_batch_destroy(lz_batch *batch, lz_stream_t stream);
  * timed trial compressions of a device-resident sample: among C in {2048,
  * 4096, 8192, 16384} and W in {64, 128, 256, 512} whose compression ratio
  * is within 5% of the best ratio found, the smallest C that is within 10%
- * of the fastest time (less shared memory per warp, which helps a batched
- * launch over buffers of several kinds), then the fastest; min_match 3 (2
- * for 4-byte symbols), max_match 255.  The choice changes the stream (it is
+ * of the fastest time (the warps that a launch keeps resident, and with them
+ * the buffers of a batch that run at once, grow as the chunk shrinks), then
+ * the fastest; min_match 3 (2 for 4-byte symbols), max_match 255.  Trials run
+ * one warp per chunk, as large inputs do.  The choice changes the stream (it is
  * recorded in its header), never the arithmetic: the stream is exactly
  * what lz_compress produces with the chosen parameters.  Synchronous;
  * allocates and frees temporary device buffers. */

@@ -1,4 +1,4 @@
-"""Batched compression of many uneven buffers (a few persistent launches).
+"""Batched compression of many uneven buffers (a few launches).
 
 Builds the many-buffer workload (sizes log-uniform over [4 KiB, 16 MiB],
 element types drawn uniformly from 1-byte codes, 2-byte codes, float32
@@ -54,10 +54,10 @@ def make_pools(torch, pool_bytes: int = 256 << 20, seed: int = 0, device="cuda")
 def autotuned_params(codec, pools, sample_bytes: int = 8 << 20, report: list | None = None) -> list:
     """Chunk size and window per kind from ``lz_autotune_ex`` on the head of
     each kind's pool (its launch-shape choice and every trial go to
-    `report`).  One launch sizes every warp's shared memory for the largest
-    chunk of the batch, so a kind whose sample does not compress (where a
-    large chunk only saves per-chunk overhead) is held to the largest chunk
-    chosen for a kind that does compress."""
+    `report`).  The buffers of one symbol size and range of windows share a
+    launch, whose warps have the shared memory of its largest chunk, so a kind
+    whose sample does not compress (where a large chunk only saves per-chunk
+    overhead) is held to the largest chunk chosen for a kind that does."""
     out, ratios = [], []
     for k, pool in enumerate(pools):
         n = min(pool.numel(), sample_bytes)
@@ -225,10 +225,12 @@ def run(torch, codec, w: Workload, steps: int = 3, check: int = 64) -> dict:
         "decompress_per_buffer_gbs": round(n / t_dplain / 1e9, 3),
         "ratio": round(n / float(sizes.sum()), 4),
         "sizes_equal_per_buffer": bool(same),
-        # compression: one launch per class (symbol size and range of windows)
-        "launches": {"batched": 1 + len({(p.S, max(128, 1 << (p.W - 1).bit_length()))
-                                         for p in w.params}),
-                     "per_buffer": 2 * len(items)},
+        # batched compression: one sample, then per class (symbol size and range
+        # of windows) a block per chunk or the two parses the sample chooses
+        # from; a buffer alone: a block per chunk, or sample and both parses
+        "launches": {"batched": 2 + 2 * len({(p.S, max(128, 1 << (p.W - 1).bit_length()))
+                                             for p in w.params}),
+                     "per_buffer": 4 * len(items), "at_most": True},
         "graphs": "both batched runs replayed from captured CUDA graphs",
         "params": [dict(kind=KIND_NAMES[k], S=p.S, C=p.C, W=p.W, m=p.m, M=p.M)
                    for k, p in enumerate(w.params)],

@@ -1,5 +1,5 @@
 // compress_batch.cu -- the launches of a compression batch: the headers of
-// empty buffers and one launch per class of buffers.
+// empty buffers and the launches of each class of buffers.
 #include "compress_impl.cuh"
 
 namespace glz {

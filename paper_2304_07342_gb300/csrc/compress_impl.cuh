@@ -212,8 +212,8 @@ __device__ __forceinline__ void build_chains(const typename SymType<S>::T *sym,
 // of its key (its first g symbols, as for the chains), into one 32-bit word
 // of a bitmap that starts empty (a blocked Bloom filter over the keys seen
 // so far in the chunk; the word is the high half of hash x word count, so
-// the bitmap fills whatever shared memory the chains would use, about 10
-// bits per position for 4-byte symbols).  The atomic returns the word before
+// the bitmap fills whatever shared memory the parse would use, about 40
+// bits per position for 4-byte symbols at C = 8192).  The atomic returns the word before
 // the OR; a
 // position finds all its bits already set ("flagged") whenever an earlier
 // position of an earlier slab has its key.  Two positions of one slab that
@@ -1181,7 +1181,8 @@ __device__ __forceinline__ uint32_t take_ticket(const CompressArgs &A, uint32_t 
 // the shared memory would keep resident; the limits are what the register
 // file gives the warps that fit: 72 at windows up to 128 (28 warps per SM at
 // S = 2, C = 4096: 2,140 us for 256 MiB of quantization codes, 2,230 at 64
-// with spills, 2,185 at 80), 96 up to 256 (20 warps at S = 4, C = 4096: 860 us
+// with spills, 2,185 at 80; up to 24 bytes still spill in the batch kernels,
+// whose chunks carry their buffer's parameters), 96 up to 256 (20 warps at S = 4, C = 4096: 860 us
 // for 128 MiB of Markov words, 925 at 80, 936 at 104), 128 up to 512 (14 warps
 // at S = 1, C = 8192).  The chains can do with 64 but take what their slices
 // leave (256 MiB of a float field, all literals: 205 us at 64, 198 at 96).

@@ -189,8 +189,8 @@ glz::CompressSmem compress_layout(const lz_params *p, bool masks) {
   if (masks) {
     // Bit planes in place of the links and rows in place of the payload area.
     // 1-byte symbols have no literal pre-check and take no more than these:
-    // 14 KiB instead of 34 per warp at C = 8192, W = 512, 15 warps resident
-    // per SM instead of 6.  Others keep at least the chains' space (with
+    // 15,488 B instead of 34 KiB per warp at C = 8192, W = 512, 14 warps
+    // resident per SM instead of 6.  Others keep at least the chains' space (with
     // one-byte links) for the pre-check's bitmap.
     uint32_t nw = 4;  // (a batch runs small windows with 4 words)
     while (32 * nw < p->window) nw *= 2;
@@ -1092,8 +1092,9 @@ struct DevBuf {
   size_t cap = 0;
 };
 
-// The buffers of a compression batch that one launch takes: one symbol size,
-// one parse (masks or chains) and one range of windows.
+// The buffers of a compression batch that one launch takes (or two, when a
+// sample chooses between masks and chains): one symbol size, one parse and one
+// range of windows.
 struct BatchClass {
   uint32_t S = 1, nj = 4;
   bool mask = false, coop = false;
@@ -1243,8 +1244,8 @@ cudaError_t batch_sides(lz_batch *b, size_t classes, cudaStream_t st) {
   return e;
 }
 
-// A compression batch is one launch per class of buffers (BatchClass), the
-// classes side by side on streams of the batch.  One launch over everything
+// A compression batch is launched by classes of buffers (BatchClass), side by
+// side on streams of the batch, after one launch that samples all of them.  One launch over everything
 // sized every warp's slice and registers for the largest item: with 1-, 2-
 // and 4-byte requests 11 warps per SM, 34 % of issue slots used.
 lz_status batch_create_compress(lz_ctx *ctx, const lz_batch_item *items, uint32_t n,

@@ -23,8 +23,11 @@
 // What bounds it: instruction issue.  The hash chains this replaces took
 // 20 of 32 lanes and one dependent shared-memory load per hop; here every
 // instruction of the mask and match steps runs on all lanes and the loads
-// are broadcasts or 16-byte rows.  The work per position depends on the
-// window and the number of varying bits but hardly on the data.
+// are broadcasts or 16-byte rows.  The work per position grows with the
+// window's words and with the bits that vary in the chunk, up to four groups of
+// planes for 4-byte symbols, and hardly with the matches: where symbols seldom
+// repeat, the chains cost less and a sample of the data sends the launch there
+// (sample.cuh).
 #pragma once
 
 #include <cstdint>

@@ -91,8 +91,7 @@ __device__ __forceinline__ uint32_t sample_piece(const BufDesc &B, uint32_t c, u
 }
 
 // Do the symbols of a launch seldom repeat, so that chains (of window class NW)
-// cost less than
-// masks of NW words?  A mask's cost grows with its words and with the bits in
+// cost less than masks of NW words?  A mask's cost grows with its words and with the bits in
 // which symbols differ, a chain's with the candidates.  The lines lie between
 // these, candidates per position (32 MiB in us, chains against masks):
 //   S = 4, W = 256: text 0.53, 31 bits: 169, 423; codes 7.0, 5 bits: 756, 222
